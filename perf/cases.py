@@ -201,6 +201,7 @@ def _step_state(case, d, s):
         s["kv"].len = s["len"].data_ptr()
         s["io"] = ph.HostIO(host_in, dev_in, dev_out, s["host_out"], in_split=at_in[4], out_split=at_out[-1])
     k_new, v_new, q, _, q_chunk = inputs
+    s["k_new"], s["v_new"], s["q"], s["q_chunk"] = k_new, v_new, q, q_chunk
     s["out"], s["lse"], s["out_chunk"] = outputs[0], outputs[1] if case["lse"] else None, outputs[-1]
     s["args"] = ph.make_step_args(s["kv"], k_new, v_new, q, s["out"], dh ** -0.5, s["w"], int(case["out_major"]), s["U"], n,
                                   chunks=s["ckv"], q_chunk=q_chunk, out_chunk=s["out_chunk"], Nc=Nc, scale_chunk=dh ** -0.5,
@@ -333,3 +334,131 @@ def tolerance(case):
     rel, most = {"step": (2.8e-3, 1.3e-2), "step_host": (2.8e-3, 1.3e-2), "teacher": (2.1e-3, 1.2e-2),
                  "decoder": (3.8e-3, 1.9e-2), "prefill": (3.8e-3, 1.9e-2), "advance": (6.2e-3, 2.9e-2)}[case["kind"]]
     return {"rel": 4 * rel, "max": 4 * most}
+
+
+# ---- the same in 64 bits -----------------------------------------------------------------------------------------------
+
+
+def exact(case, seed):
+    """What run() returns, from plain torch in 64 bits, with no rounding between the input and an output."""
+    Hq, Hkv, dh, P, C, D, F = _shape(case)
+    n, kind = case["n"], case["kind"]
+    s = prepare(case, seed)
+    torch.cuda.synchronize()
+    scale, om = s["scale"], case["out_major"]
+    if kind in ("step", "step_host"):
+        k, v, seg_k, seg_v = _append(case, s, s["k_new"], s["v_new"])
+        out, lse = _attend(s["q"], seg_k, seg_v, s["len0"] + 1, scale, *_prefix(s))
+        U = _matmul(out.reshape(n, D), s["w"], om).view(n, P, D)
+        if s["bias"] is not None:
+            U = U + s["bias"].double().view(P, D)
+        oc, _ = _attend(s["q_chunk"], s["kc"], s["vc"], s["clen"], scale)
+        lens = s["len0"] + 1
+        if kind == "step_host":
+            return [[out, lse, oc] if case["lse"] else [out, oc], U, lens, k, v]
+        return [out, lse if case["lse"] else None, U, oc, lens, k, v]
+    if kind == "teacher":
+        return [_causal(s["x"].double(), s["kc"], s["vc"], s["clen"], scale)]
+    if kind == "advance":
+        a = _matmul(_norm(s["latents"].double(), s["gamma"]), s["w_chunker"], om) + s["b_chunker"].double()
+        seen = {}
+
+        def attend(q, k_new, v_new):
+            seen["k"], seen["v"], seg_k, seg_v = _append(case, s, k_new, v_new)
+            return _attend(q, seg_k, seg_v, s["len0"] + 1, scale)[0]
+
+        x = _layer_exact(a, s["encoder"], s["len0"], case, attend)
+        U = _matmul(x, s["w"], om)
+        y, kc, vc = _prefill_exact(U.view(n * P, D), s["decoder"], case, s, scale)
+        return [a, x, U.view(n, P, D), y.view(n, P, D), s["len0"] + 1, seen["k"], seen["v"], torch.full_like(s["clen"], P), kc, vc]
+    if kind == "prefill":
+        y, kc, vc = _prefill_exact(s["x"].double().view(n * P, D), s["layer"], case, s, scale)
+        return [y.view(n, P, D), torch.full_like(s["clen"], P), kc, vc]
+    kc, vc, at = s["kc"].double(), s["vc"].double(), torch.arange(n, device="cuda")
+
+    def attend(q, k_new, v_new):
+        kc[at, :, s["clen0"].long()], vc[at, :, s["clen0"].long()] = k_new, v_new
+        return _attend(q, kc, vc, s["clen0"] + 1, scale)[0]
+
+    y = _layer_exact(s["x"].double(), s["layer"], s["clen0"], case, attend)
+    return [y, s["clen0"] + 1, kc, vc]
+
+
+def _matmul(x, w, out_major):
+    w = w.double()
+    return x @ (w.T if out_major else w)
+
+
+def _norm(x, gamma):
+    return x * torch.rsqrt((x * x).mean(-1, keepdim=True) + 1e-5) * gamma.double()
+
+
+def _append(case, s, k_new, v_new):
+    """The cache with one more row per sequence: as it is stored, and by sequence [n, Hkv, rows, dh]."""
+    n, at = case["n"], torch.arange(case["n"], device="cuda")
+    k, v, row = s["k"].double(), s["v"].double(), s["len0"].long()
+    if not case["paged"]:
+        k[at, :, row], v[at, :, row] = k_new.double(), v_new.double()
+        return k, v, k, v
+    page = s["table"].long()[at, row // PAGE]
+    k[page, :, row % PAGE], v[page, :, row % PAGE] = k_new.double(), v_new.double()
+    flat = lambda t: t[s["table"].long()].transpose(1, 2).reshape(n, t.shape[1], -1, t.shape[3])
+    return k, v, flat(k), flat(v)
+
+
+def _prefix(s):
+    keep = s["kv"]._keep
+    return () if keep[3] is None else (keep[3], keep[4])
+
+
+def _attend(q, k, v, length, scale, k_shared=None, v_shared=None):
+    """q [n, Hq, dh] over rows < length of k, v [n, Hkv, rows, dh] and, before them, a prefix of all: (out, log-sum-exp)."""
+    n, Hq, dh = q.shape
+    Hkv = k.shape[1]
+    q, k, v = q.double().reshape(n, Hkv, Hq // Hkv, dh), k.double(), v.double()
+    logit = torch.einsum("nhgd,nhsd->nhgs", q, k) * scale
+    logit.masked_fill_((torch.arange(k.shape[2], device=q.device) >= length[:, None]).view(n, 1, 1, -1), float("-inf"))
+    if k_shared is not None:
+        k_shared, v_shared = k_shared[0].double(), v_shared[0].double()
+        logit = torch.cat([torch.einsum("nhgd,hsd->nhgs", q, k_shared) * scale, logit], -1)
+    lse = torch.logsumexp(logit, -1)
+    p = torch.exp(logit - lse[..., None])
+    out = torch.einsum("nhgs,nhsd->nhgd", p[..., p.shape[-1] - k.shape[2]:], v)
+    if k_shared is not None:
+        out = out + torch.einsum("nhgs,hsd->nhgd", p[..., :k_shared.shape[1]], v_shared)
+    return out.reshape(n, Hq, dh), lse.reshape(n, Hq)
+
+
+def _causal(q, k, v, length, scale):
+    """q [n, rows, Hq, dh]: position t sees rows 0..t; a position that does not exist is zero."""
+    out = torch.empty_like(q)
+    for t in range(q.shape[1]):
+        out[:, t] = _attend(q[:, t], k[:, :, :t + 1], v[:, :, :t + 1], torch.full_like(length, t + 1), scale)[0]
+    return out * (torch.arange(q.shape[1], device=q.device) < length[:, None])[:, :, None, None]
+
+
+def _layer_exact(x, layer, pos, case, attend):
+    Hq, Hkv, dh, _, _, D, F = _shape(case)
+    g1, wqkv, wo, g2, wgu, wdown = layer._keep
+    om, rows = case["out_major"], x.shape[0]
+    qkv = _matmul(_norm(x, g1), wqkv, om).view(rows, Hq + 2 * Hkv, dh)
+    angle = pos.double()[:, None] * 10000.0 ** (-torch.arange(dh // 2, device="cuda", dtype=torch.float64) * 2 / dh)
+    c, sn = angle.cos()[:, None], angle.sin()[:, None]
+    a, b = qkv[:, :Hq + Hkv, :dh // 2], qkv[:, :Hq + Hkv, dh // 2:]
+    qk = torch.cat([a * c - b * sn, b * c + a * sn], -1)
+    h = x + _matmul(attend(qk[:, :Hq], qk[:, Hq:], qkv[:, Hq + Hkv:]).reshape(rows, D), wo, om)
+    gu = _matmul(_norm(h, g2), wgu, om)
+    return h + _matmul(torch.nn.functional.silu(gu[:, :F]) * gu[:, F:], wdown, om)
+
+
+def _prefill_exact(x, layer, case, s, scale):
+    Hq, Hkv, dh, P, _, _, _ = _shape(case)
+    n = case["n"]
+    kc, vc = s["kc"].double(), s["vc"].double()
+
+    def attend(q, k_new, v_new):
+        kc[:, :, :P], vc[:, :, :P] = (t.view(n, P, Hkv, dh).transpose(1, 2) for t in (k_new, v_new))
+        full = torch.full((n,), P, dtype=torch.int32, device="cuda")
+        return _causal(q.reshape(n, P, Hq, dh), kc[:, :, :P], vc[:, :, :P], full, scale)
+
+    return _layer_exact(x, layer, torch.arange(P, device="cuda").repeat(n), case, attend), kc, vc
