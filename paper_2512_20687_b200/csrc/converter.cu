@@ -47,9 +47,13 @@ struct ConvTile {
     static constexpr int extra = BM * BK * 2 + 1024 + 512;
 };
 
-__host__ __device__ inline int conv_stages(int ring_bytes, int a_bytes, int b_bytes, int ka) {
+// A multiple of the MMA warps: each of them then meets the same stages turn after turn, every phase of their barriers.
+// With two warps and an odd count a warp would come back to a stage only every second phase, and its wait for the
+// later phase, of the same parity as its last one, would be met by that one while the other warp's load of the
+// stage is still in flight (loads land out of order): a stage read too early, and one arrival too many on `empty`.
+__host__ __device__ constexpr int conv_stages(int ring_bytes, int a_bytes, int b_bytes, int ka, int mma_warps) {
     const int s = ring_bytes / (ka * (a_bytes + b_bytes));
-    return s < MAX_STAGES ? s : MAX_STAGES;
+    return (s < MAX_STAGES ? s : MAX_STAGES) / mma_warps * mma_warps;
 }
 
 // The loops of the TMA warp and of the MMA warp are run by the whole warp (so that their
@@ -70,7 +74,7 @@ converter_umma_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm
     uint8_t *gen = smem_raw + (base - ptx::smem_u32(smem_raw));
     const int a_bytes = p.x_rows * BK * 2;                       // x atom of this launch
     const int stage_bytes = KA * (a_bytes + T::B_BYTES);         // [x atoms][weight atoms]
-    const int n_stages = conv_stages(RING, a_bytes, T::B_BYTES, KA);
+    const int n_stages = conv_stages(RING, a_bytes, T::B_BYTES, KA, mma_warps<NT>());
     constexpr int TAIL = RING + BM * BK * 2;
     const uint32_t bars = base + TAIL;                           // full[s] +16s, empty[s] +16s+8
     const uint32_t bar_acc = bars + 16 * MAX_STAGES;

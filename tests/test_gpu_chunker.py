@@ -90,6 +90,24 @@ def test_linear_with_more_tiles_than_sms_repeated_on_an_idle_device():
             assert torch.equal(y.view(torch.int16), y0.view(torch.int16))
 
 
+@pytest.mark.parametrize("B", [1, 16])
+def test_linear_of_few_rows_and_a_long_ring(B):
+    """At most 16 rows make the ring's stages smallest, and 88 blocks of K turn it several times over: repeated calls give
+    one result, that of torch in 32 bits (half a bf16 step of values below 8, and the order of the sums)."""
+    K, N = 5632, 4864
+    x = dev_bf16(wl.normal_bf16(27, "x", (B, K)))
+    w = dev_bf16(wl.normal_bf16(27, "w", (K, N), std=K ** -0.5))
+    want = x.double() @ w.double()
+    with Ctx(cfg_small(0)) as c:
+        y0, y = (torch.empty((B, N), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        ph.photon_linear(c.h, x, w, ph.PHOTON_W_IN_MAJOR, None, y0)
+        for _ in range(40):
+            ph.photon_linear(c.h, x, w, ph.PHOTON_W_IN_MAJOR, None, y)
+            assert c.status() == 0
+            assert torch.equal(y.view(torch.int16), y0.view(torch.int16))
+    assert (y0.double() - want).abs().max() <= 2.0 ** -6 + 1e-4
+
+
 def test_large_tile_kernel_adds_bias_and_residual_and_is_deterministic(oracle):
     """Thousands of rows with bias and a residual that aliases the output; the oracle
     recomputes a sample of rows; two calls give the same bits."""
