@@ -74,6 +74,7 @@ struct AttnParams {
     int upc;                 // filled by the launcher: units per CTA on shared keys
     int own_rows;            // filled by the launcher: the units' own keys (at most this many rows each) are read by the
                              // shared-prefix kernel, which then writes the final result; 0: a second kernel reads them
+    bool over_bus;           // chunk attention: queries and results lie in host memory
     float scale_log2;        // scale * log2(e): logits are kept in the base-2 domain
     float *partials;
     float *cta_partials;
@@ -112,7 +113,8 @@ struct ConvParams {
     int B, D, N;             // N = P * D
     int w_out_major;
     int x_rows;              // filled by the launcher: x rows fetched per K block (16, 32, 64 or 128)
-    int ksplit;              // CTAs (one cluster) sharing an output tile, each on a slice of K; 0 or 1: none
+    int ksplit;              // filled by the launcher: CTAs (one cluster) sharing an output tile, each on a slice of K
+    int stages;              // filled by the launcher: stages of the ring
     int32_t *status;
 };
 
@@ -182,7 +184,7 @@ cudaError_t launch_chunk_attention(photon_ctx *ctx, const AttnParams &p, cudaStr
                                    long long *launches);
 cudaError_t launch_chunk_causal_attention(photon_ctx *ctx, const CausalParams &p, cudaStream_t st,
                                           long long *launches);
-cudaError_t launch_linear(photon_ctx *ctx, ConvParams p, cudaStream_t st, long long *launches);
+cudaError_t launch_linear(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches);
 bool linear_wants_large_tiles(const photon_ctx *ctx, const ConvParams &p);
 cudaError_t launch_linear_large(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches);
 cudaError_t launch_gate_up_large(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches);
@@ -197,8 +199,6 @@ cudaError_t launch_rope_split_append(const bf16 *qkv, int n, int Hq, int Hkv, in
                                      bf16 *v_cache, int32_t *len, int cap, Paging pg, int32_t *status, cudaStream_t st,
                                      long long *launches);
 cudaError_t launch_swiglu(const bf16 *gu, bf16 *out, int n, int F, cudaStream_t st, long long *launches);
-cudaError_t launch_converter(photon_ctx *ctx, const ConvParams &p, cudaStream_t st,
-                             long long *launches);
 cudaError_t launch_read_probe(photon_ctx *ctx, const void *src, size_t bytes, int ctas, unsigned int *sum_out,
                               cudaStream_t st, long long *launches);
 cudaError_t launch_wait_probe(photon_ctx *ctx, unsigned long long limit_ns, cudaStream_t st, long long *launches);

@@ -1,405 +1,409 @@
 // Context converter U^(l) (Section 2.1.2): U[b, n] = sum_k x[b,k] W[k,n] (+ bias[n]),
-// n = r*D + j for prefix r, feature j.
+// n = r*D + j for prefix r, feature j; and every other projection y = x W (+ b) (+ residual)
+// of up to some hundreds of rows (K and N multiples of 64): the context chunker's, the layers'.
 //
-// A dense contraction on the 5th-generation tensor cores.  A CTA owns a
-// [128 batch rows x NT output columns] tile of U: the batch rows are the M
-// side, a slab of NT weight columns is the N side, and the accumulator lives
-// in TMEM.  Only as many x rows as the batch needs (rounded up to 16, 32, 64 or
-// 128) are fetched per K block; the MMA still spans 128 rows, and the rows it
-// reads beyond the fetched ones are whatever shared memory holds: they only
-// reach accumulator rows that are never read back.  A smaller x box makes a
-// stage smaller, so a small batch gets a deeper ring of weight tiles in flight.
-// One warp feeds a ring of TMA loads (x atoms and weight atoms for 128 K
-// elements per stage), one warp issues tcgen05.mma on the swizzled atoms (in both
-// an elected lane does the issuing), four warps read the accumulator back with
-// tcgen05.ld, add the bias, round once to bf16 and store.  Every weight element leaves HBM exactly once; at small batch the
-// kernel is bound by that stream, at large batch by the tensor pipe.
+// At these sizes the weights are most of what is read, so the kernel is built around their stream.
+// The output is cut into tiles of 128 batch rows x NT weight columns, and the K range of a tile over
+// a thread-block cluster of ksplit CTAs, so that about every SM holds a CTA with an equal share of the
+// weights (the launcher's rule is beside it).  A CTA has a TMA ring whose stages hold one or two blocks of 64
+// K elements: of the NT weight columns, and of the x rows the batch needs.  Weights and x are issued by a
+// warp each: the weight half of the whole ring is requested before the dependency wait, because weights
+// never come from the kernel before.  The contraction is tcgen05.mma (batch rows on the M side, fp32 in
+// TMEM); an MMA spans 128 rows, what it reads beyond the fetched ones only reaches accumulator rows that
+// nobody reads.
 //
-// The same kernel serves any y = x W + b with K and N multiples of 64 (the
-// context chunker's linear map, Section 2.1.1: K = C_L * D, N = D).  When N is
-// so small that the output tiles would leave most SMs without a share of the
-// weight stream, the K range of a tile is split over the CTAs of a thread-block
-// cluster: each accumulates its slice, the others stage their fp32 tile in
-// their (by then free) ring and send it to the first CTA's ring with one bulk
-// copy through distributed shared memory; that CTA adds the tiles in rank order,
-// so the result does not depend on timing.
+// A split tile is put together by reduce-scatter: the tile's columns are dealt to the CTAs of the
+// cluster in groups of 16; every CTA stages the groups of the others in its (by then free) ring, one
+// bulk copy per peer moves them through distributed shared memory, and each CTA adds what it received
+// to its own groups in rank order (the result does not depend on timing), adds bias and residual,
+// rounds once and stores.
+//
+// GATED: the gate/up projection of the MLP with its activation folded in.  W is [gate | up] with N = 2F
+// columns; a tile is NT/2 gate columns and the NT/2 up columns of the same features, and silu(gate) * up goes
+// into U [B, F] (both rounded to bf16 first, as when they are stored and read back by the activation
+// kernel).  No bias, no residual.
+#include <algorithm>
+#include <type_traits>
+
 #include "common.cuh"
 #include "ptx.cuh"
 
 namespace {
 
-constexpr int BM = 128;                 // batch rows per CTA (UMMA M)
-constexpr int BK = 64;                  // K elements per swizzle atom (one 128-byte row)
-template <int NT> __host__ __device__ constexpr int atoms_per_stage() { return NT >= 256 ? 1 : 2; }   // 128 (64) K elements per barrier round trip
-constexpr int CONV_THREADS = 224;       // warp 0: TMA, warps 1 and 6: MMA (1 owns TMEM), warps 2-5: epilogue
-// With narrow weight slabs two warps issue MMAs: they take alternate stages and accumulate into
-// separate TMEM columns, because issuing a tcgen05.mma costs one thread more time than a narrow
-// MMA takes to run; the epilogue adds the accumulators.  Wide slabs gain nothing from it.
-template <int NT> __host__ __device__ constexpr int mma_warps() { return NT <= 64 ? 2 : 1; }
-
+constexpr int BM = 128;                 // batch rows per tile (UMMA M)
+constexpr int BK = 64;                  // K elements per block (one 128-byte swizzled row)
+constexpr int SLAB_THREADS = 256;       // warp 0: weights, 1 and 7: MMA (1 owns TMEM), 6: x; then all eight: epilogue
+// Blocks per stage.  A stage costs its issuers and the MMA warp a round trip to a barrier (95 cycles) and more beside
+// the copies and MMAs themselves (48 to 64 cycles each for narrow tiles): with one block per stage that paced tiles of 64
+// columns at 200 ns per block, whatever was loaded.
+__host__ __device__ constexpr int blocks_per_stage(int nt) { return nt <= 128 ? 2 : 1; }
+// Tiles of 64 columns have two MMA warps, on alternate stages and with an accumulator each (the epilogue adds them), so that
+// one's barrier and commit (36 cycles) pass under the other's MMAs: with one, the drain of a ring that was filled ahead of the
+// dependency wait is 1.2 us longer (converter of 64 rows, 2048 -> 8192, inside the decode step).  The stages are then a
+// multiple of the MMA warps: each warp meets every phase of the barriers it waits for.
+__host__ __device__ constexpr int mma_warps(int nt) { return nt == 64 ? 2 : 1; }
 constexpr int MAX_STAGES = 12;
-constexpr int RING_BYTES = 192 * 1024;  // one CTA per SM; more output tiles than SMs run as further waves
+constexpr int GROUP = 16;               // accumulator columns that change hands together
+constexpr int QUAD_BYTES = 32 * GROUP * 4;          // a group's values of 32 rows
+constexpr int BAR_BYTES = 512;
+constexpr int RING_BYTES = 208 * 1024;
 
-template <int NT>
-struct ConvTile {
-    static constexpr int B_BYTES = NT * BK * 2;           // weight atom: 8 / 16 KiB
-    // slack after the ring: the MMA reads 128 rows from every x atom, also past a short x box
-    static constexpr int extra = BM * BK * 2 + 1024 + 512;
-};
+// First group of the part of a tile that CTA r of ks puts together.
+__host__ __device__ __forceinline__ int first_group(int groups, int r, int ks) { return groups * r / ks; }
 
-// A multiple of the MMA warps: each of them then meets the same stages turn after turn, every phase of their barriers.
-// With two warps and an odd count a warp would come back to a stage only every second phase, and its wait for the
-// later phase, of the same parity as its last one, would be met by that one while the other warp's load of the
-// stage is still in flight (loads land out of order): a stage read too early, and one arrival too many on `empty`.
-__host__ __device__ constexpr int conv_stages(int ring_bytes, int a_bytes, int b_bytes, int ka, int mma_warps) {
-    const int s = ring_bytes / (ka * (a_bytes + b_bytes));
-    return (s < MAX_STAGES ? s : MAX_STAGES) / mma_warps * mma_warps;
+__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
+    __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<uint32_t *>(&t);
 }
 
-// The loops of the TMA warp and of the MMA warp are run by the whole warp (so that their
-// address arithmetic stays warp-uniform); one elected lane issues the asynchronous operations.
-// GATED (slabs of 128 columns only): the gate/up projection of the MLP with its activation folded in.  W is
-// [gate | up] with N = 2F columns; a CTA takes 64 gate columns and the 64 up columns of the same features, and
-// writes silu(gate) * up for them into U [B, F] (both projections rounded to bf16 first, as when they are
-// stored and read back by the activation kernel).  No bias, no residual, no split of K.
-template <int NT, bool W_IN_MAJOR, bool SPLIT, bool GATED = false>
-__global__ void __launch_bounds__(CONV_THREADS, 1)
-converter_umma_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
-                      const __grid_constant__ CUtensorMap tm_w) {
-    using T = ConvTile<NT>;
-    constexpr int KA = atoms_per_stage<NT>();
-    constexpr int RING = RING_BYTES;
-    extern __shared__ uint8_t smem_raw[];
-    const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
-    uint8_t *gen = smem_raw + (base - ptx::smem_u32(smem_raw));
-    const int a_bytes = p.x_rows * BK * 2;                       // x atom of this launch
-    const int stage_bytes = KA * (a_bytes + T::B_BYTES);         // [x atoms][weight atoms]
-    const int n_stages = conv_stages(RING, a_bytes, T::B_BYTES, KA, mma_warps<NT>());
-    constexpr int TAIL = RING + BM * BK * 2;
-    const uint32_t bars = base + TAIL;                           // full[s] +16s, empty[s] +16s+8
-    const uint32_t bar_acc = bars + 16 * MAX_STAGES;
-    const uint32_t bar_rx = bar_acc + 8;                         // split K: the other CTAs' tiles have landed here
-    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(gen + TAIL + 16 * MAX_STAGES + 16);
+// n groups of this warp's 32 rows from the accumulator (both: the sum of two); GATED: group g is 8 gate columns and the 8
+// up columns of the same features.
+template <int NT, bool GATED, int n>
+__device__ __forceinline__ void load_groups(uint32_t acc, bool both, int g, uint32_t (&r)[n * GROUP]) {
+    if constexpr (GATED) {
+#pragma unroll
+        for (int h = 0; h < n; ++h) {
+            ptx::tmem_ld_32x8(acc + (g + h) * (GROUP / 2), r + h * GROUP);
+            ptx::tmem_ld_32x8(acc + NT / 2 + (g + h) * (GROUP / 2), r + h * GROUP + GROUP / 2);
+        }
+    } else {
+#pragma unroll
+        for (int h = 0; h < n; ++h) ptx::tmem_ld_32x16(acc + (g + h) * GROUP, r + h * GROUP);
+    }
+    if constexpr (mma_warps(NT) == 2) {
+        uint32_t r2[n * GROUP];
+#pragma unroll
+        for (int h = 0; h < n; ++h) ptx::tmem_ld_32x16(acc + NT + (g + h) * GROUP, r2 + h * GROUP);
+        ptx::tmem_ld_wait();
+        if (both)
+#pragma unroll
+            for (int e = 0; e < n * GROUP; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) + __uint_as_float(r2[e]));
+    } else {
+        ptx::tmem_ld_wait();
+    }
+}
+
+template <int NT, bool W_IN_MAJOR, bool GATED>
+__global__ void __launch_bounds__(SLAB_THREADS, 1)
+linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w) {
+    constexpr int W_BYTES = NT * BK * 2, GROUPS = NT / GROUP, KA = blocks_per_stage(NT), MW = mma_warps(NT);
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const uint32_t base = ptx::smem_u32(smem_raw);
+    const int x_bytes = p.x_rows * BK * 2;
+    const uint32_t w_base = base + p.stages * KA * x_bytes;      // all x blocks first: an MMA reads past the end of a short one
+    const uint32_t full = base + RING_BYTES, empty = full + 8 * MAX_STAGES;
+    const uint32_t bar_acc = empty + 8 * MAX_STAGES, bar_rx = bar_acc + 8;   // accumulator complete; peers' groups landed
+    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem_raw + RING_BYTES + 16 * MAX_STAGES + 16);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int ks = SPLIT ? p.ksplit : 1;                         // CTAs (one cluster) that share an output tile
-    const int zr = ks > 1 ? (int)(blockIdx.x % ks) : 0;          // = rank in the cluster: which slice of K
-    static_assert(!GATED || (NT == 128 && !SPLIT), "the gated form takes 64 gate and 64 up columns, whole K");
+    const int ks = p.ksplit, zr = (int)(blockIdx.x % ks);        // zr = rank in the cluster: which slice of K
     const int n0 = (int)(blockIdx.x / ks) * (GATED ? NT / 2 : NT), m0 = blockIdx.y * BM;
-    const int up0 = p.N / 2 + n0;                                // GATED: first of this CTA's up columns
-    constexpr int MMA_WARPS = mma_warps<NT>();
-    const uint32_t stg_bytes = (uint32_t)p.x_rows * NT * 4;      // the fetched rows of one fp32 tile, stored [column][row]
+    const int up0 = p.N / 2 + n0;                                // GATED: first of this tile's up columns
     const int a_lo = (p.D / BK) * zr / ks, n_atoms = (p.D / BK) * (zr + 1) / ks - a_lo;
     const int n_steps = (n_atoms + KA - 1) / KA;
+    const int nq = p.x_rows > 32 ? p.x_rows / 32 : 1;            // quarters of the tile's rows that hold batch rows
+    const int g_lo = first_group(GROUPS, zr, ks), own = first_group(GROUPS, zr + 1, ks) - g_lo;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < n_stages; ++s) {
-            ptx::mbar_init(bars + 16 * s, 1);
-            ptx::mbar_init(bars + 16 * s + 8, 1);
+        for (int s = 0; s < p.stages; ++s) {
+            ptx::mbar_init(full + 8 * s, 2);                     // two issuers, each with its own bytes
+            ptx::mbar_init(empty + 8 * s, 1);
         }
-        ptx::mbar_init(bar_acc, MMA_WARPS);
+        ptx::mbar_init(bar_acc, MW);
         ptx::mbar_init(bar_rx, 1);
         ptx::mbar_fence_init();
-        if (ks > 1 && zr == 0) ptx::mbar_arrive_expect_tx(bar_rx, (ks - 1) * stg_bytes);
+        if (ks > 1) ptx::mbar_arrive_expect_tx(bar_rx, (ks - 1) * own * nq * QUAD_BYTES);
         ptx::prefetch_tmap(&tm_x); ptx::prefetch_tmap(&tm_w);
     }
-    if (warp == 1) ptx::tmem_alloc(ptx::smem_u32(const_cast<uint32_t *>(tmem_slot)), MMA_WARPS * NT);
+    if (warp == 1) ptx::tmem_alloc(ptx::smem_u32(const_cast<uint32_t *>(tmem_slot)), MW * NT);
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    ptx::grid_dep_launch();                 // one CTA per SM; the next kernel lines up once the last wave has started
+    ptx::grid_dep_launch();
 
-    // The weights never come from the kernel before this one, x may: the ring's first turn requests its
-    // weight atoms at once and its x atoms once the dependency wait has returned, so that the weight stream
-    // already runs under the tail of the predecessor.  The same thread issues both, after it has told the
-    // stage's barrier how many bytes to expect: were another warp to issue the x atoms, then with no
-    // predecessor in flight (calls launched one by one) an x atom could land before its stage's byte count is
-    // posted.  Everything else this kernel does with global memory follows from x having landed.
-    auto load_x = [&](int st, int s) {
-        const int atoms = min(KA, n_atoms - st * KA);
-        const uint32_t a_dst = base + s * stage_bytes;
-        for (int j = 0; j < atoms; ++j)
-            ptx::tma_load_2d(a_dst + j * a_bytes, &tm_x, (a_lo + st * KA + j) * BK, m0, bars + 16 * s);   // x[m0.., k0..]
-    };
-    const int ahead = min(n_steps, n_stages);              // the ring starts empty: no stage to wait for
-
-    if (warp == 0) {
-        auto load_w = [&](int st, int s) {
-            const int atoms = min(KA, n_atoms - st * KA);
-            const uint32_t full = bars + 16 * s;
-            const uint32_t b_dst = base + s * stage_bytes + KA * a_bytes;
-            for (int j = 0; j < atoms; ++j) {
+    // One lane of each of these warps does the work; there is nothing to vote on.
+    if (warp != 0) ptx::grid_dep_wait();                         // x may be the output of the kernel before this one
+    if ((warp == 0 || warp == 6) && ptx::elect_one()) {
+        int s = 0;
+        for (int st = 0; st < n_steps; ++st) {
+            if (st >= p.stages && !ptx::mbar_wait(empty + 8 * s, (st / p.stages - 1) & 1)) {
+                atomicOr(p.status, PHOTON_DEV_TIMEOUT);
+                break;
+            }
+            const int n = min(KA, n_atoms - st * KA);
+            const uint32_t bar = full + 8 * s;
+            ptx::mbar_arrive_expect_tx(bar, n * (warp == 6 ? x_bytes : W_BYTES));
+#pragma unroll
+            for (int j = 0; j < KA; ++j) {
+                if (j >= n) break;
                 const int k0 = (a_lo + st * KA + j) * BK;
+                if (warp == 6) {
+                    ptx::tma_load_2d(base + (s * KA + j) * x_bytes, &tm_x, k0, m0, bar);     // x[m0.., k0..]
+                    continue;
+                }
+                const uint32_t dst = w_base + (s * KA + j) * W_BYTES;
                 if (!W_IN_MAJOR) {
-                    if (GATED) {                                                         // two boxes of 64 rows: gate, then up
-                        ptx::tma_load_2d(b_dst + j * T::B_BYTES, &tm_w, k0, n0, full);
-                        ptx::tma_load_2d(b_dst + j * T::B_BYTES + 64 * 128, &tm_w, k0, up0, full);
-                    } else {
-                        ptx::tma_load_2d(b_dst + j * T::B_BYTES, &tm_w, k0, n0, full);   // W[n0.., k0..]  (K-major)
-                    }
+                    ptx::tma_load_2d(dst, &tm_w, k0, n0, bar);                           // W[n0.., k0..]  (K-major)
+                    if (GATED) ptx::tma_load_2d(dst + W_BYTES / 2, &tm_w, k0, up0, bar);
                 } else {
 #pragma unroll
-                    for (int jj = 0; jj < NT / 64; ++jj)                                 // W[k0.., n0+64jj..] (N-major)
-                        ptx::tma_load_2d(b_dst + j * T::B_BYTES + jj * (BK * 128), &tm_w,
-                                         GATED ? (jj == 0 ? n0 : up0) : n0 + 64 * jj, k0, full);
+                    for (int jj = 0; jj < NT / 64; ++jj)                                 // W[k0.., n..] (N-major), 64 columns a box
+                        ptx::tma_load_2d(dst + jj * (BK * 128), &tm_w,
+                                         GATED ? (jj < NT / 128 ? n0 + 64 * jj : up0 + 64 * (jj - NT / 128)) : n0 + 64 * jj, k0, bar);
                 }
             }
-        };
-        if (ptx::elect_one())
-            for (int st = 0; st < ahead; ++st) {
-                ptx::mbar_arrive_expect_tx(bars + 16 * st, min(KA, n_atoms - st * KA) * (a_bytes + T::B_BYTES));
-                load_w(st, st);
-            }
-        __syncwarp();
-        ptx::grid_dep_wait();               // x may be the output of the kernel before this one
-        if (ptx::elect_one())
-            for (int st = 0; st < ahead; ++st) load_x(st, st);
-        __syncwarp();
-        int s = ahead == n_stages ? 0 : ahead;
-        uint32_t phase = ahead == n_stages ? 1 : 0;
-        for (int st = ahead; st < n_steps; ++st) {
-            if (!__all_sync(0xffffffffu, ptx::mbar_wait(bars + 16 * s + 8, phase ^ 1))) {
-                if (lane == 0) atomicOr(p.status, PHOTON_DEV_TIMEOUT);
-                break;
-            }
-            if (ptx::elect_one()) {
-                ptx::mbar_arrive_expect_tx(bars + 16 * s, min(KA, n_atoms - st * KA) * (a_bytes + T::B_BYTES));
-                load_x(st, s);
-                load_w(st, s);
-            }
-            __syncwarp();
-            if (++s == n_stages) { s = 0; phase ^= 1; }
+            if (++s == p.stages) s = 0;
         }
-    } else if (warp == 1 || (warp == 6 && MMA_WARPS == 2)) {
+    } else if ((warp == 1 || (MW == 2 && warp == 7)) && ptx::elect_one()) {
         constexpr uint32_t idesc = ptx::umma_idesc_bf16(BM, NT, false, W_IN_MAJOR);
-        const int me = warp == 1 ? 0 : 1;                  // which accumulator, and which stages
-        const uint32_t acc = tmem + me * NT;
-        const int last_mine = n_steps - 1 >= me ? n_steps - 1 - ((n_steps - 1 - me) % MMA_WARPS) : -1;
-        int s = 0;
+        const int me = warp == 1 ? 0 : 1;                        // which stages, which accumulator
+        int s = me;
         uint32_t phase = 0;
-        bool first = true;
-        if (last_mine < 0 && ptx::elect_one()) ptx::mbar_arrive(bar_acc);      // fewer steps than MMA warps
-        for (int st = 0; st < n_steps; ++st) {
-            if (st % MMA_WARPS != me) {
-                if (++s == n_stages) { s = 0; phase ^= 1; }
-                continue;
-            }
-            if (!__all_sync(0xffffffffu, ptx::mbar_wait(bars + 16 * s, phase))) {
-                if (lane == 0) atomicOr(p.status, PHOTON_DEV_TIMEOUT);
+        if (me >= n_steps) ptx::mbar_arrive(bar_acc);            // fewer steps than MMA warps
+        for (int st = me; st < n_steps; st += MW) {
+            if (!ptx::mbar_wait(full + 8 * s, phase)) {
+                atomicOr(p.status, PHOTON_DEV_TIMEOUT);
                 break;
             }
-            ptx::tc_fence_after();
-            const int atoms = min(KA, n_atoms - st * KA);
-            const uint32_t a_addr = base + s * stage_bytes, b_addr = a_addr + KA * a_bytes;
-            if (ptx::elect_one()) {
-                for (int j = 0; j < atoms; ++j) {
-                    const uint64_t adesc = ptx::umma_desc_sw128(a_addr + j * a_bytes, 0, 1024);
-                    const uint64_t bdesc = W_IN_MAJOR ? ptx::umma_desc_sw128(b_addr + j * T::B_BYTES, BK * 128, 1024)
-                                                      : ptx::umma_desc_sw128(b_addr + j * T::B_BYTES, 0, 1024);
+            const int n = min(KA, n_atoms - st * KA);
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k) {
-                        // advance 16 K elements: 32 bytes inside the swizzled row (K-major),
-                        // 16 rows of 128 bytes (N-major); the address field counts 16-byte units
-                        const uint64_t a_k = adesc + (uint64_t)(k * 2);
-                        const uint64_t b_k = bdesc + (uint64_t)(W_IN_MAJOR ? k * 128 : k * 2);
-                        ptx::umma_bf16(acc, a_k, b_k, idesc, !first || (j | k) != 0);
-                    }
-                }
-                ptx::umma_commit(bars + 16 * s + 8);       // frees the stage once these MMAs have read it
-                if (st == last_mine) ptx::umma_commit(bar_acc);       // this warp's accumulator is complete
+            for (int j = 0; j < KA; ++j) {
+                if (j >= n) break;
+                const uint64_t adesc = ptx::umma_desc_sw128(base + (s * KA + j) * x_bytes, 0, 1024);
+                const uint64_t bdesc = ptx::umma_desc_sw128(w_base + (s * KA + j) * W_BYTES, W_IN_MAJOR ? BK * 128 : 0, 1024);
+#pragma unroll
+                for (int k = 0; k < BK / 16; ++k)
+                    // advance 16 K elements: 32 bytes inside the swizzled row (K-major),
+                    // 16 rows of 128 bytes (N-major); the address field counts 16-byte units
+                    ptx::umma_bf16(tmem + me * NT, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(W_IN_MAJOR ? k * 128 : k * 2), idesc,
+                                   st != me || (j | k) != 0);
             }
-            first = false;
-            __syncwarp();
-            if (++s == n_stages) { s = 0; phase ^= 1; }
+            ptx::umma_commit(st + MW >= n_steps ? bar_acc : empty + 8 * s); // frees the stage once these MMAs have read it
+            s += MW;
+            if (s >= p.stages) { s -= p.stages; phase ^= 1; }
         }
     }
-    // epilogue: warp w (2..5) reads TMEM lanes [32*(w%4), +32) = batch rows m0 + that range
-    const bool epi = warp >= 2 && warp <= 5;
-    const int quad = warp & 3;
-    bool ok = true;
-    if (epi) {
-        ok = ptx::mbar_wait(bar_acc, 0);
-        if (!ok && lane == 0) atomicOr(p.status, PHOTON_DEV_TIMEOUT);
-        ptx::tc_fence_after();
-        ptx::grid_dep_wait();               // long since over; these warps read the residual and write the output
+    __syncwarp();
+
+    if (warp == 0) ptx::grid_dep_wait();                         // (the weights did not wait; what follows does)
+
+    // ---- epilogue: warp w reads TMEM lanes [32*(w%4), +32) = batch rows m0 + that range, half of the groups each:
+    // one warp per scheduler is bound by the latency of its own instructions, so all eight take part
+    const int quad = warp & 3, half = warp >> 2;
+    const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16);
+    const bool both = n_steps > 1;          // (with one step the second accumulator is untouched)
+    bool ok = ptx::mbar_wait(bar_acc, 0);
+    if (!ok && lane == 0) atomicOr(p.status, PHOTON_DEV_TIMEOUT);
+    __syncwarp();
+    ptx::tc_fence_after();
+    const uint32_t recv = base + (GROUPS - GROUPS / ks) * nq * QUAD_BYTES;       // behind the largest staging area of any rank
+    if (ks > 1) {
+        ptx::cluster_arrive();                             // this CTA's ring is free
+        if (quad < nq)
+            for (int g = 2 * half; g < GROUPS; g += 4) {   // the other CTAs' groups, in the order of their owners
+                uint32_t r[2 * GROUP];
+                load_groups<NT, GATED, 2>(acc, both, g, r);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (g + h >= g_lo && g + h < g_lo + own) continue;
+                    const uint32_t at = base + ((g + h < g_lo ? g + h : g + h - own) * nq + quad) * QUAD_BYTES + lane * 16;
+#pragma unroll
+                    for (int j = 0; j < GROUP / 4; ++j)
+                        ptx::sts128(at + j * 512, make_uint4(r[GROUP * h + 4 * j], r[GROUP * h + 4 * j + 1], r[GROUP * h + 4 * j + 2],
+                                                             r[GROUP * h + 4 * j + 3]));
+                }
+            }
+        ptx::fence_proxy_async();                          // the staged groups are read by bulk copies
+        __syncthreads();
+        ptx::cluster_wait();                               // every CTA's ring is free: groups may land there
+        if (warp == 2 && lane < ks && lane != zr) {
+            // lane -> peer: its groups of this CTA's tile, to the place of this rank in the peer's receive area
+            const int lo = first_group(GROUPS, lane, ks), cnt = first_group(GROUPS, lane + 1, ks) - lo;
+            const uint32_t bytes = cnt * nq * QUAD_BYTES;
+            ptx::bulk_copy_to_peer(ptx::map_cluster(recv + (zr < lane ? zr : zr - 1) * bytes, lane),
+                                   base + (lo < g_lo ? lo : lo - own) * nq * QUAD_BYTES, bytes, ptx::map_cluster(bar_rx, lane));
+        }
+        __syncwarp();
     }
-    if (ks > 1) ptx::cluster_sync();        // every CTA of the cluster is done with its ring
-    if (epi) {
-        const int row = quad * 32 + lane, b = m0 + row;
-        if (ks > 1 && zr == 0) {
-            const bool got = ptx::mbar_wait(bar_rx, 0);
+    if (quad < nq) {
+        const int b = m0 + quad * 32 + lane;
+        const bool live = b < p.B;
+        const int mid = g_lo + (own + 1) / 2;              // groups [g_lo, mid) are the first four warps', the rest the others'
+        int g = half ? mid : g_lo;
+        const int end = half ? g_lo + own : mid;
+        // whole sectors where the output's alignment allows it (16 bytes are all that the caller owes, and a gated pair
+        // that starts at an odd group starts in the middle of a sector)
+        const bool wide = (reinterpret_cast<uintptr_t>(p.U) & 31u) == 0 && !(GATED && (g & 1));
+        if (ks > 1) {
+            const bool got = __all_sync(0xffffffffu, ptx::mbar_wait(bar_rx, 0));
             if (!got && lane == 0) atomicOr(p.status, PHOTON_DEV_TIMEOUT);
             ok = ok && got;
         }
-        if constexpr (GATED) {
-            const int F = p.N / 2;
-#pragma unroll 1
-            for (int c0 = 0; c0 < NT / 2; c0 += 32) {
-                uint32_t g[32], u[32];
-                ptx::tmem_ld_32x32(tmem + ((uint32_t)(quad * 32) << 16) + c0, g);
-                ptx::tmem_ld_32x32(tmem + ((uint32_t)(quad * 32) << 16) + NT / 2 + c0, u);
-                ptx::tmem_ld_wait();
-                if (ok && b < p.B) {
-                    uint4 *dst = reinterpret_cast<uint4 *>(p.U + (size_t)b * F + n0 + c0);
+        // groups [g, g + n): own accumulator + the other slices in rank order, then bias, residual, rounding
+        auto finish = [&](auto n_tag, int g) {
+            constexpr int n = decltype(n_tag)::value, COLS = n * GROUP, WORDS = GATED ? COLS / 4 : COLS / 2;
+            __syncwarp();                                  // rows past the batch left the round before early
+            uint32_t r[COLS], res[COLS / 2], w[WORDS];
+            const int col = n0 + g * GROUP;
+            if (!GATED && p.residual && live)
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        uint32_t w[4];
+                for (int v = 0; v < COLS / 8; ++v) {
+                    const uint4 u = __ldcg(reinterpret_cast<const uint4 *>(p.residual + (size_t)b * p.N + col) + v);
+                    res[4 * v] = u.x; res[4 * v + 1] = u.y; res[4 * v + 2] = u.z; res[4 * v + 3] = u.w;
+                }
+            load_groups<NT, GATED, n>(acc, both, g, r);
+            for (int z = 0; z < ks - 1; ++z)
+#pragma unroll
+                for (int h = 0; h < n; ++h) {
+                    const uint32_t at = recv + ((z * own + g + h - g_lo) * nq + quad) * QUAD_BYTES + lane * 16;
+#pragma unroll
+                    for (int j = 0; j < GROUP / 4; ++j) {
+                        const uint4 v = ptx::lds128(at + j * 512);
+                        uint32_t *d = r + h * GROUP + 4 * j;
+                        d[0] = __float_as_uint(__uint_as_float(d[0]) + __uint_as_float(v.x));
+                        d[1] = __float_as_uint(__uint_as_float(d[1]) + __uint_as_float(v.y));
+                        d[2] = __float_as_uint(__uint_as_float(d[2]) + __uint_as_float(v.z));
+                        d[3] = __float_as_uint(__uint_as_float(d[3]) + __uint_as_float(v.w));
+                    }
+                }
+            if (!live || !ok) return;
+            bf16 *dst;
+            if constexpr (GATED) {
+#pragma unroll
+                for (int e = 0; e < WORDS; ++e) {          // group h: 8 gate values, then the 8 up values of the same features
+                    const int h = e / (GROUP / 4), i = h * GROUP + 2 * (e % (GROUP / 4));
+                    const float g0 = __bfloat162float(__float2bfloat16_rn(__uint_as_float(r[i])));
+                    const float g1 = __bfloat162float(__float2bfloat16_rn(__uint_as_float(r[i + 1])));
+                    const float u0 = __bfloat162float(__float2bfloat16_rn(__uint_as_float(r[GROUP / 2 + i])));
+                    const float u1 = __bfloat162float(__float2bfloat16_rn(__uint_as_float(r[GROUP / 2 + i + 1])));
+                    w[e] = pack2(g0 / (1.f + __expf(-g0)) * u0, g1 / (1.f + __expf(-g1)) * u1);
+                }
+                dst = p.U + (size_t)b * (p.N / 2) + n0 + g * (GROUP / 2);
+            } else {
+                if (p.residual)
+#pragma unroll
+                    for (int e = 0; e < WORDS; ++e) {
+                        r[2 * e] = __float_as_uint(__uint_as_float(r[2 * e]) + bf16_lo(res[e]));
+                        r[2 * e + 1] = __float_as_uint(__uint_as_float(r[2 * e + 1]) + bf16_hi(res[e]));
+                    }
+                if (p.bias)
+#pragma unroll
+                    for (int v = 0; v < COLS / 8; ++v) {
+                        const uint4 bv = __ldcg(reinterpret_cast<const uint4 *>(p.bias + col) + v);
+                        const uint32_t bw[4] = {bv.x, bv.y, bv.z, bv.w};
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            const float g0 = __bfloat162float(__float2bfloat16_rn(__uint_as_float(g[v * 8 + 2 * e])));
-                            const float g1 = __bfloat162float(__float2bfloat16_rn(__uint_as_float(g[v * 8 + 2 * e + 1])));
-                            const float u0 = __bfloat162float(__float2bfloat16_rn(__uint_as_float(u[v * 8 + 2 * e])));
-                            const float u1 = __bfloat162float(__float2bfloat16_rn(__uint_as_float(u[v * 8 + 2 * e + 1])));
-                            __nv_bfloat162 o = __floats2bfloat162_rn(g0 / (1.f + __expf(-g0)) * u0, g1 / (1.f + __expf(-g1)) * u1);
-                            w[e] = *reinterpret_cast<uint32_t *>(&o);
+                            r[8 * v + 2 * e] = __float_as_uint(__uint_as_float(r[8 * v + 2 * e]) + bf16_lo(bw[e]));
+                            r[8 * v + 2 * e + 1] = __float_as_uint(__uint_as_float(r[8 * v + 2 * e + 1]) + bf16_hi(bw[e]));
                         }
-                        dst[v] = make_uint4(w[0], w[1], w[2], w[3]);
                     }
+#pragma unroll
+                for (int e = 0; e < WORDS; ++e) w[e] = pack2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1]));
+                dst = p.U + (size_t)b * p.N + col;
+            }
+            if constexpr (WORDS >= 8) {
+                if (wide) {
+#pragma unroll
+                    for (int v = 0; v < WORDS; v += 8) ptx::stg256(dst + 2 * v, w + v);
+                    return;
                 }
             }
-        } else {
-#pragma unroll 1
-        for (int c0 = 0; c0 < NT; c0 += 32) {
-            uint32_t r[32];
-            ptx::tmem_ld_32x32(tmem + ((uint32_t)(quad * 32) << 16) + c0, r);
-            ptx::tmem_ld_wait();
-            if (MMA_WARPS == 2 && n_steps > 1) {           // second accumulator (untouched when there is one step)
-                uint32_t r2[32];
-                ptx::tmem_ld_32x32(tmem + ((uint32_t)(quad * 32) << 16) + NT + c0, r2);
-                ptx::tmem_ld_wait();
 #pragma unroll
-                for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) + __uint_as_float(r2[e]));
-            }
-            if (zr != 0) {                                 // stage this slice's tile for the first CTA
-                if (row < p.x_rows) {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        *reinterpret_cast<uint32_t *>(gen + ((size_t)(c0 + e) * p.x_rows + row) * 4) = r[e];
-                }
-                continue;
-            }
-            for (int z = 1; z < ks && row < p.x_rows; ++z) {   // add the other slices in rank order
-                const float *part = reinterpret_cast<const float *>(gen + (size_t)(z - 1) * stg_bytes);
-#pragma unroll
-                for (int e = 0; e < 32; ++e)
-                    r[e] = __float_as_uint(__uint_as_float(r[e]) + part[(size_t)(c0 + e) * p.x_rows + row]);
-            }
-            if (ok && b < p.B) {
-                uint4 *dst = reinterpret_cast<uint4 *>(p.U + (size_t)b * p.N + n0 + c0);
-                const uint4 *res = p.residual ? reinterpret_cast<const uint4 *>(p.residual + (size_t)b * p.N + n0 + c0) : nullptr;
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    uint32_t w[4];
-                    const uint4 rv = res ? __ldcg(res + v) : make_uint4(0u, 0u, 0u, 0u);
-                    const uint32_t rw[4] = {rv.x, rv.y, rv.z, rv.w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        float f0 = __uint_as_float(r[v * 8 + 2 * e]) + bf16_lo(rw[e]);
-                        float f1 = __uint_as_float(r[v * 8 + 2 * e + 1]) + bf16_hi(rw[e]);
-                        if (p.bias) {
-                            f0 += __bfloat162float(p.bias[n0 + c0 + v * 8 + 2 * e]);
-                            f1 += __bfloat162float(p.bias[n0 + c0 + v * 8 + 2 * e + 1]);
-                        }
-                        __nv_bfloat162 t = __floats2bfloat162_rn(f0, f1);
-                        w[e] = *reinterpret_cast<uint32_t *>(&t);
-                    }
-                    dst[v] = make_uint4(w[0], w[1], w[2], w[3]);
-                }
-            }
-        }
-        }                                                  // (not GATED)
-        if (zr != 0) {
-            ptx::fence_proxy_async();                      // the staged tile is read by the bulk copy
-            ptx::named_bar_sync(1, 128);                   // the four epilogue warps
-            if (warp == 2 && ptx::elect_one())
-                ptx::bulk_copy_to_peer(ptx::map_cluster(base + (uint32_t)(zr - 1) * stg_bytes, 0), base, stg_bytes,
-                                       ptx::map_cluster(bar_rx, 0));
-        }
+            for (int v = 0; v < WORDS; v += 4) *reinterpret_cast<uint4 *>(dst + 2 * v) = make_uint4(w[v], w[v + 1], w[v + 2], w[v + 3]);
+        };
+        for (; g + 2 <= end; g += 2) finish(std::integral_constant<int, 2>{}, g);
+        if (g < end) finish(std::integral_constant<int, 1>{}, g);
     }
-    if (ks > 1) ptx::cluster_sync();        // the first CTA has every tile: the senders' rings may go
     ptx::tc_fence_before();
-    __syncthreads();
+    if (ks > 1) ptx::cluster_sync();        // every CTA has received its groups: the senders' shared memory may go
+    else __syncthreads();
     if (warp == 1) {
         ptx::tc_fence_after();
-        ptx::tmem_dealloc(tmem, MMA_WARPS * NT);
+        ptx::tmem_dealloc(tmem, MW * NT);
     }
 }
 
-template <int NT, bool IN_MAJOR, bool SPLIT, bool GATED = false>
-cudaError_t run_as(photon_ctx *ctx, const ConvParams &p, const CUtensorMap &mx, const CUtensorMap &mw, dim3 grid,
-                   cudaStream_t st) {
-    using T = ConvTile<NT>;
-    constexpr size_t smem = (size_t)RING_BYTES + T::extra;
+// How a projection is cut: NT columns per tile, ks CTAs per tile, and the ring stages that fit.
+struct SlabPlan {
+    int nt, ks, stages;
+};
+
+// The cut with the least estimated time, from measurements (one call after another, weights from HBM; microseconds):
+// a block of 64 K elements takes a CTA 0.165 / 0.25 / 0.37 for a tile of 64 / 128 / 256 columns, never less than the
+// weights take at 4.6 TB/s over the whole grid; a wave of CTAs adds 2; an exchange 0.6, and 0.4 and the time of its
+// bytes at 30 KB a microsecond per further CTA of the cluster.  So K is split only as far as the exchange is
+// cheaper than the blocks it saves: 127 x 2048 -> 2048 takes 7.8 unsplit, 6.7 as 32 tiles x 4 and 7.8 as 16 tiles
+// x 4; 127 x 5632 -> 2048 17.1, 9.5 and 11.5; 1204 x 2048 -> 2048 15.2 as 80 tiles of 256 columns, 18.7 as 160 of
+// 128 (two waves).
+SlabPlan slab_plan(const photon_ctx *ctx, int B, int K, int N, int x_rows, bool gated) {
+    const int m_tiles = (B + BM - 1) / BM, atoms = K / BK, nq = x_rows > 32 ? x_rows / 32 : 1;
+    const float weights_us = (float)N * K * 2 / 4.6e6f;
+    SlabPlan best{};
+    float best_us = 0.f;
+    for (int nt = 64; nt <= 256; nt *= 2) {
+        if (N % nt != 0 || (gated && nt != 128)) continue;
+        const int groups = nt / GROUP;
+        const float block_us = nt == 64 ? 0.165f : nt == 128 ? 0.25f : 0.37f;
+        for (int ks = 1; ks <= 8 && ks <= groups && ks * 2 <= std::max(2, atoms); ++ks) {
+            const int own_lo = groups / ks, own_hi = (groups + ks - 1) / ks;
+            const int send = (groups - own_lo) * nq * QUAD_BYTES, recv = (ks - 1) * own_hi * nq * QUAD_BYTES;
+            if (ks > 1 && send + recv > RING_BYTES) continue;
+            const long long ctas = (long long)(N / nt) * m_tiles * ks, waves = (ctas + ctx->sm_count - 1) / ctx->sm_count;
+            const float us = std::max((float)waves * ((atoms + ks - 1) / ks) * block_us, weights_us) + 2.f * waves +
+                             (ks > 1 ? 0.6f + 0.4f * (ks - 1) + send / 30e3f : 0.f);
+            if (best.nt == 0 || us < best_us) {
+                const int stages = std::min(MAX_STAGES, RING_BYTES / (blocks_per_stage(nt) * (x_rows + nt) * BK * 2));
+                best = SlabPlan{nt, ks, stages / mma_warps(nt) * mma_warps(nt)};
+                best_us = us;
+            }
+        }
+    }
+    return best;
+}
+
+template <int NT, bool IN_MAJOR, bool GATED>
+cudaError_t run_as(photon_ctx *ctx, ConvParams p, const SlabPlan &s, cudaStream_t st, long long *launches) {
+    const CUtensorMap *t;
+    CUtensorMap mx, mw;
+    if (!(t = ctx->tmaps.get(p.x, (uint64_t)p.B, (uint64_t)p.D, p.x_rows))) return cudaErrorInvalidValue;
+    mx = *t;
+    // [K, N] in boxes of 64 k x 64 n, or [N, K] in boxes of NT n x 64 k (gate rows and up rows are fetched apart)
+    t = IN_MAJOR ? ctx->tmaps.get(p.w, (uint64_t)p.D, (uint64_t)p.N, BK) : ctx->tmaps.get(p.w, (uint64_t)p.N, (uint64_t)p.D, GATED ? NT / 2 : NT);
+    if (!t) return cudaErrorInvalidValue;
+    mw = *t;
+    p.ksplit = s.ks; p.stages = s.stages;
+    constexpr size_t smem = (size_t)RING_BYTES + BAR_BYTES;
     static size_t smem_set[kMaxDevices] = {};
-    if (const cudaError_t e = ensure_dynamic_smem(converter_umma_kernel<NT, IN_MAJOR, SPLIT, GATED>, smem, ctx->device, smem_set)) return e;
-    return launch_dependent(converter_umma_kernel<NT, IN_MAJOR, SPLIT, GATED>, grid, dim3(CONV_THREADS), smem, st,
-                            p.ksplit > 1 ? p.ksplit : 0, p, mx, mw);
-}
-
-// out [B, F] = silu(x Wg) * (x Wu) for w = [Wg | Wu] (N = 2F columns), 64 features per CTA.
-template <bool IN_MAJOR>
-cudaError_t run_gated(photon_ctx *ctx, ConvParams p, cudaStream_t st, long long *launches) {
-    p.x_rows = p.B > 64 ? 128 : p.B > 32 ? 64 : p.B > 16 ? 32 : 16;
-    p.ksplit = 1;
-    const CUtensorMap *t;
-    CUtensorMap mx, mw;
-    if (!(t = ctx->tmaps.get(p.x, (uint64_t)p.B, (uint64_t)p.D, p.x_rows))) return cudaErrorInvalidValue;
-    mx = *t;
-    // [K, N] in boxes of 64 k x 64 n, or [N, K] in boxes of 64 n x 64 k (gate rows and up rows are fetched apart)
-    t = IN_MAJOR ? ctx->tmaps.get(p.w, (uint64_t)p.D, (uint64_t)p.N, BK) : ctx->tmaps.get(p.w, (uint64_t)p.N, (uint64_t)p.D, 64);
-    if (!t) return cudaErrorInvalidValue;
-    mw = *t;
-    const dim3 grid(p.N / 128, (p.B + BM - 1) / BM);
-    const cudaError_t e = run_as<128, IN_MAJOR, false, true>(ctx, p, mx, mw, grid, st);
+    if (const cudaError_t e = ensure_dynamic_smem(linear_slab_kernel<NT, IN_MAJOR, GATED>, smem, ctx->device, smem_set)) return e;
+    const dim3 grid(p.ksplit * (p.N / NT), (p.B + BM - 1) / BM);
+    const cudaError_t e = launch_dependent(linear_slab_kernel<NT, IN_MAJOR, GATED>, grid, dim3(SLAB_THREADS), smem, st,
+                                           p.ksplit > 1 ? p.ksplit : 0, p, mx, mw);
     ++*launches;
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <int NT, bool IN_MAJOR>
+template <bool GATED>
 cudaError_t run(photon_ctx *ctx, ConvParams p, cudaStream_t st, long long *launches) {
+    if (p.B == 0) return cudaSuccess;
     p.x_rows = p.B > 64 ? 128 : p.B > 32 ? 64 : p.B > 16 ? 32 : 16;
-    const CUtensorMap *t;
-    CUtensorMap mx, mw;
-    if (!(t = ctx->tmaps.get(p.x, (uint64_t)p.B, (uint64_t)p.D, p.x_rows))) return cudaErrorInvalidValue;
-    mx = *t;
-    if (IN_MAJOR) t = ctx->tmaps.get(p.w, (uint64_t)p.D, (uint64_t)p.N, BK);        // [K, N], boxes of 64 k x 64 n
-    else t = ctx->tmaps.get(p.w, (uint64_t)p.N, (uint64_t)p.D, NT);                 // [N, K], boxes of NT n x 64 k
-    if (!t) return cudaErrorInvalidValue;
-    mw = *t;
-    if (p.ksplit < 1) p.ksplit = 1;
-    dim3 grid(p.ksplit * (p.N / NT), (p.B + BM - 1) / BM);
-    cudaError_t e;
-    if constexpr (NT == 64)
-        e = p.ksplit > 1 ? run_as<NT, IN_MAJOR, true>(ctx, p, mx, mw, grid, st) : run_as<NT, IN_MAJOR, false>(ctx, p, mx, mw, grid, st);
-    else
-        e = run_as<NT, IN_MAJOR, false>(ctx, p, mx, mw, grid, st);
-    ++*launches;
-    return e != cudaSuccess ? e : cudaGetLastError();
+    const SlabPlan s = slab_plan(ctx, p.B, p.D, p.N, p.x_rows, GATED);
+    if constexpr (GATED) {
+        if (s.nt != 128) return cudaErrorInvalidValue;
+        return p.w_out_major ? run_as<128, false, true>(ctx, p, s, st, launches) : run_as<128, true, true>(ctx, p, s, st, launches);
+    } else {
+        if (p.w_out_major)
+            return s.nt == 256 ? run_as<256, false, false>(ctx, p, s, st, launches)
+                               : s.nt == 128 ? run_as<128, false, false>(ctx, p, s, st, launches) : run_as<64, false, false>(ctx, p, s, st, launches);
+        return s.nt == 256 ? run_as<256, true, false>(ctx, p, s, st, launches)
+                           : s.nt == 128 ? run_as<128, true, false>(ctx, p, s, st, launches) : run_as<64, true, false>(ctx, p, s, st, launches);
+    }
 }
 
 }  // namespace
 
-// y = x W + b for any K (p.D) and N that are multiples of 64.  Few output tiles: narrow slabs, then the
-// K range split over clusters of 2 or 4 CTAs, as long as a CTA keeps at least 8 K blocks of 64.
-cudaError_t launch_linear(photon_ctx *ctx, ConvParams p, cudaStream_t st, long long *launches) {
-    if (p.B == 0) return cudaSuccess;
-    const int m_tiles = (p.B + BM - 1) / BM;
-    const bool wide = p.B > 128 && p.N % 128 == 0 && (p.N / 128) * m_tiles * 2 >= ctx->sm_count;
-    const bool wider = wide && p.N % 256 == 0 && (p.N / 256) * m_tiles >= 100;
-    // narrow slabs that would need a second wave of CTAs: twice as wide, one wave
-    const bool second_wave = !wide && p.N % 128 == 0 && (long long)(p.N / 64) * m_tiles > ctx->sm_count &&
-                             (long long)(p.N / 128) * m_tiles <= ctx->sm_count;
-    const int nt = wider ? 256 : (wide || second_wave) ? 128 : 64;
-    p.ksplit = 1;
-    if (nt == 64)
-        while (p.ksplit < 4 && (p.N / nt) * m_tiles * p.ksplit * 2 <= ctx->sm_count && (p.D / BK) / (p.ksplit * 2) >= 8)
-            p.ksplit *= 2;
-    if (p.w_out_major)
-        return nt == 256 ? run<256, false>(ctx, p, st, launches)
-                         : nt == 128 ? run<128, false>(ctx, p, st, launches) : run<64, false>(ctx, p, st, launches);
-    return nt == 256 ? run<256, true>(ctx, p, st, launches)
-                     : nt == 128 ? run<128, true>(ctx, p, st, launches) : run<64, true>(ctx, p, st, launches);
+cudaError_t launch_linear(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches) {
+    return run<false>(ctx, p, st, launches);
 }
 
 // Whether the fused gate/up form serves this shape: whole slabs of 64 features, and enough of them to occupy most
@@ -410,20 +414,5 @@ bool gate_up_fits_small_tiles(const photon_ctx *ctx, const ConvParams &p) {
 }
 
 cudaError_t launch_gate_up(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches) {
-    if (p.B == 0) return cudaSuccess;
-    return p.w_out_major ? run_gated<false>(ctx, p, st, launches) : run_gated<true>(ctx, p, st, launches);
-}
-
-cudaError_t launch_converter(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches) {
-    if (p.B == 0) return cudaSuccess;
-    // wider weight slabs once the batch is large enough for the tensor pipe to matter, as long as
-    // about one CTA per SM remains
-    const int m_tiles = (p.B + BM - 1) / BM;
-    const bool wide = p.B > 128 && p.N % 128 == 0;
-    const bool wider = wide && p.N % 256 == 0 && (p.N / 256) * m_tiles >= 100;
-    if (p.w_out_major)
-        return wider ? run<256, false>(ctx, p, st, launches)
-                     : wide ? run<128, false>(ctx, p, st, launches) : run<64, false>(ctx, p, st, launches);
-    return wider ? run<256, true>(ctx, p, st, launches)
-                 : wide ? run<128, true>(ctx, p, st, launches) : run<64, true>(ctx, p, st, launches);
+    return run<true>(ctx, p, st, launches);
 }
