@@ -108,6 +108,30 @@ def test_linear_of_few_rows_and_a_long_ring(B):
     assert (y0.double() - want).abs().max() <= 2.0 ** -6 + 1e-4
 
 
+@pytest.mark.parametrize("B,K,N", [(1, 64, 64), (17, 192, 128), (33, 1024, 320), (64, 8192, 2048), (127, 2048, 2048), (129, 448, 256),
+                                   (256, 5632, 2048), (600, 2048, 3072)])
+@pytest.mark.parametrize("out_major", [False, True])
+def test_projection_cuts_and_outputs_that_are_only_16_byte_aligned(B, K, N, out_major):
+    """One block of K, ragged rows and slices of K, tiles of 64, 128 and 256 columns, clusters of one to several CTAs; output,
+    residual and bias 16 bytes into their allocations.  Against torch in 64 bits: half a bf16 step of the result (2^-8 of
+    its magnitude, or of one where it is smaller) and the rounding of sums of K products in 32 bits."""
+    g = torch.Generator("cuda").manual_seed(B + K + N)
+
+    def new(*shape, std=1.0):
+        n = int(np.prod(shape))
+        return (torch.randn(n + 8, generator=g, device="cuda") * std).to(torch.bfloat16)[8:].view(*shape)
+
+    x, w, bias, res = new(B, K), new(K, N, std=K ** -0.5), new(N), new(B, N)
+    want = x.double() @ w.double() + bias.double() + res.double()
+    y = new(B, N)
+    assert y.data_ptr() % 32 == 16
+    with Ctx(cfg_small(0)) as c:
+        layout = ph.PHOTON_W_OUT_MAJOR if out_major else ph.PHOTON_W_IN_MAJOR
+        ph.photon_linear(c.h, x, w.t().contiguous() if out_major else w, layout, bias, y, residual=res)
+        assert c.status() == 0
+    assert ((y.double() - want).abs() <= 2.0 ** -8 * want.abs().clamp(min=1.0) + 1e-4).all()
+
+
 def test_large_tile_kernel_adds_bias_and_residual_and_is_deterministic(oracle):
     """Thousands of rows with bias and a residual that aliases the output; the oracle
     recomputes a sample of rows; two calls give the same bits."""
