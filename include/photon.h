@@ -222,7 +222,7 @@ photon_status photon_linear(photon_ctx *ctx, const photon_bf16 *x, const photon_
  * caller owns the intermediates in `scratch` (sizes beside the fields); each
  * is rounded to bf16 where the next kernel reads it.  y may alias x.  Where
  * the gate/up projection's slabs of 64 features occupy at least half of the
- * GPU's SMs (F / 64 slabs per 128 rows), and with thousands of rows, that
+ * GPU's SMs (F / 64 slabs per 128 rows), and with many rows, that
  * projection and the activation are one launch and scratch->gu is left
  * unwritten (eight launches); both projections are rounded to bf16 before
  * the activation either way.

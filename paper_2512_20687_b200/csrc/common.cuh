@@ -198,9 +198,12 @@ cudaError_t launch_linear(photon_ctx *ctx, const ConvParams &p, cudaStream_t st,
 cudaError_t linear_cluster_counts(int device, int (&fit)[MAX_CLUSTER + 1]);
 // for tests: {columns per tile, CTAs per tile, ring stages, MMA warps} of a projection on a device that holds fit[ks] clusters
 void linear_cut(const int *fit, int B, int K, int N, bool gated, int32_t *cut);
-bool linear_wants_large_tiles(const photon_ctx *ctx, const ConvParams &p);
-cudaError_t launch_linear_large(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches);
-cudaError_t launch_gate_up_large(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches);
+float linear_slab_us(const int *fit, const ConvParams &p, bool gated);
+bool linear_wants_pairs(const int *fit, const ConvParams &p, bool gated);
+// for tests: {taken, columns per tile, row tiles, column tiles, whole tiles, pieces, ring stages, bytes per stage}
+void linear_pair_cut(const int *fit, const ConvParams &p, bool gated, int32_t *cut);
+cudaError_t launch_linear_pairs(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches);
+cudaError_t launch_gate_up_pairs(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches);
 bool gate_up_fits_small_tiles(const photon_ctx *ctx, const ConvParams &p);
 cudaError_t launch_gate_up(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches);
 // registers of a CTA as it is allocated: the 64-column projection's, and the register chunk attention's (128 features,

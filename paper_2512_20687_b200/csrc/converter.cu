@@ -220,6 +220,23 @@ linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
     const int quad = warp & 3, half = warp >> 2;
     const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16);
     const bool both = n_steps > 1;          // (with one step the second accumulator is untouched)
+    const int b = m0 + quad * 32 + lane;
+    const bool live = quad < nq && b < p.B;
+    const int mid = g_lo + (own + 1) / 2;   // groups [g_lo, mid) are the first four warps', the rest the others'
+    const int g_begin = half ? mid : g_lo, g_end = half ? g_lo + own : mid;
+    // the residual of the next groups to finish, requested well before it is added: a trip to the L2 per round otherwise
+    // (4096 x 2048 -> 2048: 46.9 us, 42 since)
+    uint4 res[AT_ONCE * GROUP / 8];
+    auto fetch_residual = [&](int g) {
+        if constexpr (!GATED) {
+            if (!p.residual || !live) return;
+#pragma unroll
+            for (int v = 0; v < AT_ONCE * GROUP / 8; ++v)
+                if (g + v / (GROUP / 8) < g_end)
+                    res[v] = __ldcg(reinterpret_cast<const uint4 *>(p.residual + (size_t)b * p.N + n0 + g * GROUP) + v);
+        }
+    };
+    fetch_residual(g_begin);
     // one lane polls: 256 threads at the barrier hold up those that feed it (128 x 1024 -> 1024: 5.2 us, 5.0 with one)
     bool ok = lane != 0 || ptx::mbar_wait(bar_acc, 0);
     if (!ok) atomicOr(p.status, PHOTON_DEV_TIMEOUT);
@@ -256,11 +273,7 @@ linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
         __syncwarp();
     }
     if (quad < nq) {
-        const int b = m0 + quad * 32 + lane;
-        const bool live = b < p.B;
-        const int mid = g_lo + (own + 1) / 2;              // groups [g_lo, mid) are the first four warps', the rest the others'
-        int g = half ? mid : g_lo;
-        const int end = half ? g_lo + own : mid;
+        int g = g_begin;
         // whole sectors where the output's alignment allows it (16 bytes are all that the caller owes, and a gated pair
         // that starts at an odd group starts in the middle of a sector)
         const bool wide = (reinterpret_cast<uintptr_t>(p.U) & 31u) == 0 && !(GATED && (g & 1));
@@ -272,14 +285,8 @@ linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
         // groups [g, g + n): own accumulator + the other slices in rank order, then bias, residual, rounding
         auto finish = [&](auto n_tag, int g) {
             constexpr int n = decltype(n_tag)::value, COLS = n * GROUP, WORDS = GATED ? COLS / 4 : COLS / 2;
-            uint32_t r[COLS], res[COLS / 2], w[WORDS];
-            const int col = n0 + g * GROUP;
-            if (!GATED && p.residual && live)
-#pragma unroll
-                for (int v = 0; v < COLS / 8; ++v) {
-                    const uint4 u = __ldcg(reinterpret_cast<const uint4 *>(p.residual + (size_t)b * p.N + col) + v);
-                    res[4 * v] = u.x; res[4 * v + 1] = u.y; res[4 * v + 2] = u.z; res[4 * v + 3] = u.w;
-                }
+            uint32_t r[COLS], w[WORDS];
+            [[maybe_unused]] const int col = n0 + g * GROUP;
             __syncwarp();                                  // rows past the batch took no part above, and left the round before early
             load_groups<NT, GATED, n>(acc, both, g, r);
             for (int z = 0; z < ks - 1; ++z)
@@ -310,12 +317,18 @@ linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
                 }
                 dst = p.U + (size_t)b * (p.N / 2) + n0 + g * (GROUP / 2);
             } else {
-                if (p.residual)
+                if (p.residual) {
 #pragma unroll
-                    for (int e = 0; e < WORDS; ++e) {
-                        r[2 * e] = __float_as_uint(__uint_as_float(r[2 * e]) + bf16_lo(res[e]));
-                        r[2 * e + 1] = __float_as_uint(__uint_as_float(r[2 * e + 1]) + bf16_hi(res[e]));
+                    for (int v = 0; v < COLS / 8; ++v) {
+                        const uint32_t rw[4] = {res[v].x, res[v].y, res[v].z, res[v].w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            r[8 * v + 2 * e] = __float_as_uint(__uint_as_float(r[8 * v + 2 * e]) + bf16_lo(rw[e]));
+                            r[8 * v + 2 * e + 1] = __float_as_uint(__uint_as_float(r[8 * v + 2 * e + 1]) + bf16_hi(rw[e]));
+                        }
                     }
+                    fetch_residual(g + n);
+                }
                 if (p.bias)
 #pragma unroll
                     for (int v = 0; v < COLS / 8; ++v) {
@@ -341,8 +354,8 @@ linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
 #pragma unroll
             for (int v = 0; v < WORDS; v += 4) *reinterpret_cast<uint4 *>(dst + 2 * v) = make_uint4(w[v], w[v + 1], w[v + 2], w[v + 3]);
         };
-        for (; g + AT_ONCE <= end; g += AT_ONCE) finish(std::integral_constant<int, AT_ONCE>{}, g);
-        if (AT_ONCE > 1 && g < end) finish(std::integral_constant<int, 1>{}, g);
+        for (; g + AT_ONCE <= g_end; g += AT_ONCE) finish(std::integral_constant<int, AT_ONCE>{}, g);
+        if (AT_ONCE > 1 && g < g_end) finish(std::integral_constant<int, 1>{}, g);
     }
     __syncwarp();                           // (rows past the batch left the last round early: the barriers below want whole warps)
     ptx::tc_fence_before();
@@ -357,6 +370,7 @@ linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
 // How a projection is cut: NT columns per tile, ks CTAs per tile, and the ring stages that fit.
 struct SlabPlan {
     int nt, ks, stages;
+    float us;                // the estimate
 };
 
 // The cut with the least estimated time (microseconds; constants fitted to 5,000 timed cuts, 24 weight shapes x 17 batches,
@@ -373,7 +387,6 @@ SlabPlan slab_plan(const int *fit, int B, int K, int N, int x_rows, bool gated) 
     const int m_tiles = (B + BM - 1) / BM, atoms = K / BK, nq = x_rows > 32 ? x_rows / 32 : 1;
     const float weights_us = (float)N * K * 2 / 5.75e6f, few_rows = 1.f - 0.08f * (float)(BM - x_rows) / BM;
     SlabPlan best{};
-    float best_us = 0.f;
     for (int nt = 64; nt <= 256; nt *= 2) {
         if (N % nt != 0 || (gated && nt != 128)) continue;
         const int groups = nt / GROUP;
@@ -385,10 +398,9 @@ SlabPlan slab_plan(const int *fit, int B, int K, int N, int x_rows, bool gated) 
             const long long tiles = (long long)(N / nt) * m_tiles, waves = (tiles + fit[ks] - 1) / fit[ks];
             const float us = std::max((float)waves * ((atoms + ks - 1) / ks) * block_us, weights_us) +
                              waves * (1.7f + (ks > 1 ? 1.3f + 0.33f * (ks - 1) + send / 17e3f : 0.f));
-            if (best.nt == 0 || us < best_us) {
+            if (best.nt == 0 || us < best.us) {
                 const int stages = std::min(MAX_STAGES, RING_BYTES / (blocks_per_stage(nt) * (x_rows + nt) * BK * 2));
-                best = SlabPlan{nt, ks, stages / mma_warps(nt) * mma_warps(nt)};
-                best_us = us;
+                best = SlabPlan{nt, ks, stages / mma_warps(nt) * mma_warps(nt), us};
             }
         }
     }
@@ -481,6 +493,16 @@ cudaError_t linear_cluster_counts(int device, int (&fit)[MAX_CLUSTER + 1]) {
     }
     std::copy(fit, fit + MAX_CLUSTER + 1, known[device]);
     return cudaSuccess;
+}
+
+// The time of the best cut for comparison with the pair kernel; negative where there is no cut (a gated form of half slabs).
+// The estimate above was fitted to small batches; with the whole chip at work the same cuts take about a quarter longer,
+// every wave ends in an epilogue of its own, and the residual and the output move while nothing else does (5 TB/s).
+float linear_slab_us(const int *fit, const ConvParams &p, bool gated) {
+    const SlabPlan s = slab_plan(fit, p.B, p.D, p.N, rows_fetched(p.B), gated);
+    if (s.nt == 0) return -1.f;
+    const long long tiles = (long long)(p.N / s.nt) * ((p.B + BM - 1) / BM), waves = (tiles + fit[s.ks] - 1) / fit[s.ks];
+    return 1.25f * s.us + waves * (s.nt / 256.f) + (float)p.B * p.N * (p.residual ? 4 : 2) / 5e6f;
 }
 
 void linear_cut(const int *fit, int B, int K, int N, bool gated, int32_t *cut) {

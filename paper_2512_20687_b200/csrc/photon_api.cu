@@ -284,8 +284,8 @@ photon_status converter(photon_ctx *ctx, const photon_bf16 *x, const photon_bf16
     p.w_out_major = (w_layout == PHOTON_W_OUT_MAJOR);
     p.w_ahead = w_ahead;
     p.status = ctx->status;
-    const cudaError_t e = linear_wants_large_tiles(ctx, p)      // batches of more than a thousand latents
-                              ? launch_linear_large(ctx, p, static_cast<cudaStream_t>(stream), &ctx->launches)
+    const cudaError_t e = linear_wants_pairs(ctx->clusters, p, false)      // batches of many hundreds of latents
+                              ? launch_linear_pairs(ctx, p, static_cast<cudaStream_t>(stream), &ctx->launches)
                               : launch_linear(ctx, p, static_cast<cudaStream_t>(stream), &ctx->launches);
     return e == cudaSuccess ? PHOTON_OK : PHOTON_ERR_CUDA;
 }
@@ -308,9 +308,9 @@ photon_status linear(photon_ctx *ctx, const photon_bf16 *x, const photon_bf16 *w
     p.w_out_major = (w_layout == PHOTON_W_OUT_MAJOR);
     p.w_ahead = w_ahead;
     p.status = ctx->status;
-    // thousands of rows: the persistent kernel with two accumulators in TMEM; else the converter's kernel
-    const cudaError_t e = linear_wants_large_tiles(ctx, p)
-                              ? launch_linear_large(ctx, p, static_cast<cudaStream_t>(stream), &ctx->launches)
+    // many rows: the persistent kernel of CTA pairs; else the converter's kernel
+    const cudaError_t e = linear_wants_pairs(ctx->clusters, p, false)
+                              ? launch_linear_pairs(ctx, p, static_cast<cudaStream_t>(stream), &ctx->launches)
                               : launch_linear(ctx, p, static_cast<cudaStream_t>(stream), &ctx->launches);
     return e == cudaSuccess ? PHOTON_OK : PHOTON_ERR_CUDA;
 }
@@ -365,7 +365,7 @@ photon_status photon_swiglu(photon_ctx *ctx, const photon_bf16 *gu, photon_bf16 
 
 namespace {
 // gate/up projection and activation: act [rows, F] = silu(n Wg) * (n Wu).  One fused launch (gu is then not written)
-// of the large-tile kernel with thousands of rows, of the slab kernel where 64-feature slabs occupy most of the GPU;
+// of the kernel of CTA pairs with many rows, of the slab kernel where 64-feature slabs occupy most of the GPU;
 // else the projection followed by photon_swiglu.
 photon_status gate_up(photon_ctx *ctx, const photon_layer *L, const photon_layer_scratch *sc, int rows,
                       photon_stream stream) {
@@ -378,8 +378,8 @@ photon_status gate_up(photon_ctx *ctx, const photon_layer *L, const photon_layer
     p.w_out_major = (L->w_layout == PHOTON_W_OUT_MAJOR);
     p.w_ahead = true;
     p.status = ctx->status;
-    if (L->F % 128 == 0 && linear_wants_large_tiles(ctx, p)) {
-        const cudaError_t e = launch_gate_up_large(ctx, p, static_cast<cudaStream_t>(stream), &ctx->launches);
+    if (linear_wants_pairs(ctx->clusters, p, true)) {
+        const cudaError_t e = launch_gate_up_pairs(ctx, p, static_cast<cudaStream_t>(stream), &ctx->launches);
         return e == cudaSuccess ? PHOTON_OK : PHOTON_ERR_CUDA;
     }
     if (gate_up_fits_small_tiles(ctx, p)) {                                // one launch, gu is not written
@@ -720,6 +720,13 @@ photon_status photon_wait_probe(photon_ctx *ctx, int64_t limit_ns, photon_stream
 // Not part of the interface (and not in its header): for tests.
 void photon_internal_projection_cut(const int32_t *clusters, int32_t B, int32_t K, int32_t N, int32_t gated, int32_t *cut) {
     linear_cut(clusters, B, K, N, gated != 0, cut);
+}
+void photon_internal_pair_cut(const int32_t *clusters, int32_t B, int32_t K, int32_t N, int32_t out_major, int32_t residual,
+                              int32_t gated, int32_t *cut) {
+    ConvParams p{};
+    p.B = B; p.D = K; p.N = N; p.w_out_major = out_major;
+    p.residual = residual ? reinterpret_cast<const bf16 *>(cut) : nullptr;      // (only whether there is one counts)
+    linear_pair_cut(clusters, p, gated != 0, cut);
 }
 void photon_internal_clusters(const photon_ctx *ctx, int32_t *clusters) {
     for (int i = 0; i <= MAX_CLUSTER; ++i) clusters[i] = ctx->clusters[i];

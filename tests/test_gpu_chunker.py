@@ -165,6 +165,25 @@ def check_projection(B, K, N, out_major):
     assert ((y.double() - want).abs() <= 2.0 ** -8 * want.abs().clamp(min=1.0) + 1e-4).all()
 
 
+# tiles of 128, 192 and 256 columns for pairs of CTAs: whole, all in halves, the last round in halves; a last tile past N, rows that
+# end inside a warp and rows that only the first CTA of a pair has; one block of K, and K that turns the ring
+PAIRS = [(1025, 64, 3072, (128, 120, 120)), (1600, 128, 2112, (128, 119, 119)), (1027, 64, 2112, (192, 55, 55)), (4099, 64, 640, (192, 68, 68)),
+         (2050, 128, 2112, (192, 74, 124)), (3000, 704, 448, (192, 0, 72)), (1204, 1024, 2048, (192, 55, 55)), (4099, 64, 448, (256, 0, 68)),
+         (6000, 192, 1408, (256, 144, 144)), (9001, 64, 2112, (256, 296, 352)), (1990, 2048, 2048, (256, 64, 64))]
+
+
+@pytest.mark.parametrize("B,K,N,cut", PAIRS)
+@pytest.mark.parametrize("out_major", [False, True])
+def test_projection_in_every_kind_of_cut_for_pairs(B, K, N, cut, out_major):
+    """Bounds as above."""
+    with Ctx(cfg_small(0)) as c:
+        clusters, out = (ctypes.c_int32 * 9)(), (ctypes.c_int32 * 8)()
+        ph.load().photon_internal_clusters(c.h, clusters)
+        ph.load().photon_internal_pair_cut(clusters, B, K, N, int(out_major), 1, 0, out)
+        assert out[0] and (out[1], out[4], out[5]) == cut
+    check_projection(B, K, N, out_major)
+
+
 @pytest.mark.parametrize("B,K,N", [(1, 2048, 2048), (31, 2048, 2048), (97, 8192, 256), (127, 5632, 2048), (255, 2048, 11264), (1203, 5632, 2048),
                                    (300, 128, 192), (4099, 192, 2816)])
 def test_projection_of_rows_that_end_inside_a_warp(B, K, N):

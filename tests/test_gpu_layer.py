@@ -421,3 +421,41 @@ def test_gate_up_with_the_activation_and_a_split_of_k(n, Hq, F, ks, out_major):
     silu = gate * torch.sigmoid(gate)
     err = (scratch.tensors["act"].double() - silu * up).abs()
     assert (err <= 2.0 ** -7 * (1.1 * gate.abs() + silu.abs()) * up.abs() + 2.0 ** -8 * (silu * up).abs() + 1e-4).all()
+
+
+@pytest.mark.parametrize("out_major", [False, True])
+@pytest.mark.parametrize("n,F", [(1601, 1088), (2050, 1088), (5000, 704)])
+def test_gate_up_by_pairs_with_features_that_end_inside_a_tile(n, F, out_major):
+    """The gate/up projection on pairs of CTAs, whole tiles and halves, F an odd multiple of 64.  scratch.act against torch in 64
+    bits on scratch.n, with the bound of the test above."""
+    Hq, Hkv, dh = 2, 1, 64
+    D = Hq * dh
+    g = torch.Generator("cuda").manual_seed(n + F)
+
+    def rand(*shape, std=1.0):
+        return (torch.randn(*shape, generator=g, device="cuda") * std).to(torch.bfloat16)
+
+    def weight(k, m):
+        return rand(m, k, std=k ** -0.5) if out_major else rand(k, m, std=k ** -0.5)
+
+    cfg = wl.scaled(wl.CONFIGS[4], B=1, Hq=Hq, Hkv=Hkv, dh=dh, D=D)
+    wgu, one = weight(D, 2 * F), torch.ones(D, dtype=torch.bfloat16, device="cuda")
+    layer = ph.make_layer(one, weight(D, (Hq + 2 * Hkv) * dh), weight(D, D), one, wgu, weight(F, D), int(out_major), F)
+    scratch = ph.make_layer_scratch(n, Hq, Hkv, dh, F, "cuda", torch.bfloat16)
+    k = torch.zeros(n, Hkv, 4, dh, dtype=torch.bfloat16, device="cuda")
+    kv = ph.make_kv(k, torch.zeros_like(k), torch.zeros(n, dtype=torch.int32, device="cuda"))
+    x = rand(n, D)
+    y = torch.empty_like(x)
+    with Ctx(cfg, max_queries=n) as c:
+        clusters, cut = (ctypes.c_int32 * 9)(), (ctypes.c_int32 * 8)()
+        ph.load().photon_internal_clusters(c.h, clusters)
+        ph.load().photon_internal_pair_cut(clusters, n, D, 2 * F, int(out_major), 0, 1, cut)
+        assert cut[0]
+        ph.photon_decoder_step(c.h, layer, scratch, x, kv, y, scale=dh ** -0.5)
+        assert c.status() == 0
+    w = wgu.double().T if out_major else wgu.double()
+    gu = (scratch.tensors["n"].double() @ w).to(torch.bfloat16).double()
+    gate, up = gu[:, :F], gu[:, F:]
+    silu = gate * torch.sigmoid(gate)
+    err = (scratch.tensors["act"].double() - silu * up).abs()
+    assert (err <= 2.0 ** -7 * (1.1 * gate.abs() + silu.abs()) * up.abs() + 2.0 ** -8 * (silu * up).abs() + 1e-4).all()

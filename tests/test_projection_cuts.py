@@ -60,3 +60,35 @@ def test_clusters_that_the_device_does_not_hold_are_not_taken():
     for K, N in ((8192, 2048), (16384, 256), (5632, 2048)):
         assert cut(64, K, N, clusters=(0, 148, 74, 0, 0, 0, 0, 0, 0))[1] <= 2
         assert cut(64, K, N, clusters=(0, 148, 0, 0, 0, 0, 0, 0, 0))[1] == 1
+
+
+def pair_cut(B, K, N, out_major, residual=False, gated=False, clusters=B200_CLUSTERS):
+    build.build_library()
+    out = (ctypes.c_int32 * 8)()
+    ph.load().photon_internal_pair_cut((ctypes.c_int32 * 9)(*clusters), B, K, N, int(out_major), int(residual), int(gated), out)
+    return tuple(out)
+
+
+@pytest.mark.parametrize("out_major", [False, True])
+def test_every_cut_for_pairs_covers_the_output_and_fits_the_ring(out_major):
+    pairs = B200_CLUSTERS[2]
+    for B in (1, 129, 256, 257, 300, 900, 1204, 2048, 4099, 16384):
+        for K in (64, 256, 1024, 5632):
+            for N in (64, 128, 448, 1024, 1408, 2048, 2112, 3072, 11264):
+                _, nt, m_tiles, n_tiles, whole, pieces, stages, stage_bytes = pair_cut(B, K, N, out_major)
+                what = (B, K, N, nt, whole, pieces)
+                assert nt in (128, 192, 256) and m_tiles == -(-B // 256) and n_tiles == -(-N // nt), what
+                tiles = m_tiles * n_tiles
+                assert pieces == whole + 2 * (tiles - whole), what
+                # halves are the last, partly filled round, and then fit one round
+                assert whole == tiles or (whole == tiles // pairs * pairs and pieces - whole <= pairs), what
+                # x rows and the weight columns that a stage's copies bring: N-major weights come 64 columns at a time
+                columns = nt // 2 if out_major else -(-(nt // 2) // 64) * 64
+                assert stage_bytes == (128 + columns) * 128 and stage_bytes % 1024 == 0, what
+                assert 2 <= stages <= 8 and stages * stage_bytes <= 196 * 1024, what
+
+
+def test_pairs_are_taken_for_many_rows_only_and_where_the_device_holds_them():
+    for K, N in ((2048, 3072), (2048, 2048), (1024, 3072), (5632, 2048), (2048, 11264)):
+        assert pair_cut(16384, K, N, True)[0] and not pair_cut(128, K, N, True)[0]
+        assert not pair_cut(16384, K, N, True, clusters=(0, 148, 0, 0, 0, 0, 0, 0, 0))[0]
