@@ -8,7 +8,7 @@
 // lengths of the individual caches, so there is one wave and no tail.  The
 // split points are found on the device from len[] by a block-wide prefix sum;
 // a split point that falls inside a short stream moves to the nearer end of it
-// (a cut costs more than a few tiles of imbalance), long streams are cut.
+// (a cut costs more than some tiles of imbalance), long streams are cut.
 //
 // Inside a CTA one thread drives a ring of TMA loads (128-byte-swizzled boxes of
 // 32 rows, so rows past the end of a cache are not fetched; the group's query
@@ -45,10 +45,14 @@ constexpr int STAGES = 3;
 constexpr int HALF_BYTES = BN * 128;       // 64 rows x 64 elements, swizzled
 constexpr int BOX_BYTES = BOX * 128;
 constexpr int CTAS_PER_SM = 2;
-#ifndef COARSE_SNAP
-#define COARSE_SNAP 8
-#endif
-constexpr int SNAP = COARSE_SNAP;          // streams of at most this many tiles are never cut
+// Where a stream may be cut.  A cut costs 3 to 5 us at the end of a CTA (the part's stores, a fence, a ticket and the merge, a trip
+// to the L2 each); a share that is some tiles longer costs little, because the CTAs that are through leave their bandwidth to the
+// others.  77 sequences of 0 to 1000 rows, 16/4 heads: 21.7 us with streams of up to 8 tiles whole, 18.6 with 16; longer limits
+// leave long caches to too few CTAs (20 of 0 to 3000 rows: 18.5, and 20.1 with 24 tiles whole).  Boundaries close to an end of a
+// longer stream move there: 130 of 0 to 2000 rows 50.3 -> 49.7 us; with 4 and 8 tiles instead of 2, 20 x 3000 is slower (18.8, 19.3).
+constexpr int SNAP = 16;                   // streams of at most this many tiles are never cut
+constexpr int EDGE = 2;                    // others not within this many tiles of an end
+static_assert(2 * EDGE <= SNAP, "a boundary cannot be close to both ends of a stream that is cut");
 constexpr int NLEN = 768;                  // lengths of the first NLEN units are kept in shared memory
 
 template <int DH>
@@ -74,20 +78,46 @@ __device__ __forceinline__ int tiles_of(int len) { return (len + BN - 1) / BN; }
 //
 // A length is kept as it was read, clamped to [-1, cap] (-1: any negative value).  With the step's append
 // folded into this kernel (p.k_new set) a unit with room grows by the one row the kernel itself installs:
-// the keys it attends are those of the grown cache.
-__device__ __forceinline__ int ld_len(const AttnParams &p, int u) { return max(-1, min(__ldcg(p.len + u), p.cap)); }
+// the keys it attends are those of the grown cache.  A paged unit whose new row would fall into a page that does not
+// exist is kept as -2 - length: it attends what it has and does not grow.
+__device__ __forceinline__ int clamp_len(const AttnParams &p, int len) { return max(-1, min(len, p.cap)); }
 __device__ __forceinline__ bool appends(const AttnParams &p, int raw) { return p.k_new && raw >= 0 && raw < p.cap; }
-__device__ __forceinline__ int eff_len(const AttnParams &p, int raw) { return appends(p, raw) ? raw + 1 : max(raw, 0); }
+__device__ __forceinline__ int held(int raw) { return raw >= 0 ? raw : raw <= -2 ? -2 - raw : 0; }     // rows before an append
+__device__ __forceinline__ int eff_len(const AttnParams &p, int raw) { return appends(p, raw) ? raw + 1 : held(raw); }
+__device__ __forceinline__ int ld_page(const AttnParams &p, int u, int row) {
+    return __ldcg(p.page_table + (size_t)u * p.pages_per_unit + row / p.page_rows);
+}
+__device__ __forceinline__ bool page_ok(const AttnParams &p, int id) { return id >= 0 && id < p.n_pages; }
+// (PAGED is a template parameter of everything that looks at pages: beside other kernels this one's instructions come out of the L2
+// each time, and with the page look-ups in the code of contiguous caches too a step of 64 sequences took 29.5 instead of 25.4 us.)
+template <bool PAGED>
+__device__ __forceinline__ int ld_len(const AttnParams &p, int u) {
+    const int raw = clamp_len(p, __ldcg(p.len + u));
+    return PAGED && appends(p, raw) && !page_ok(p, ld_page(p, u, raw)) ? -2 - raw : raw;
+}
 
 constexpr int LPT = NLEN / THREADS;        // lengths per thread when a batch fits the shared-memory copy
 static_assert(NLEN % THREADS == 0, "a thread's units must fit its registers");
 
-// The lengths of units [ub, ue), at most LPT of them, requested before any is used.
-__device__ __forceinline__ void load_lengths(const AttnParams &p, int ub, int ue, int (&len)[LPT]) {
+// The lengths of units [ub, ue), at most LPT of them, requested before any is used; `at`: lengths to look the new rows' pages up
+// by, so that lengths and pages come in one trip (where a length turns out to differ, its page is not asked for).
+template <bool PAGED>
+__device__ __forceinline__ void load_lengths(const AttnParams &p, int ub, int ue, int (&len)[LPT], const int *at) {
+    [[maybe_unused]] int id[LPT] = {};
 #pragma unroll
     for (int i = 0; i < LPT; ++i) len[i] = ub + i < ue ? __ldcg(p.len + ub + i) : 0;
+    if (PAGED && p.k_new) {
 #pragma unroll
-    for (int i = 0; i < LPT; ++i) len[i] = max(-1, min(len[i], p.cap));
+        for (int i = 0; i < LPT; ++i) {
+            const int row = ub + i >= ue ? -1 : at ? held(at[ub + i]) : clamp_len(p, len[i]);
+            if (row >= 0 && row < p.cap) id[i] = ld_page(p, ub + i, row);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < LPT; ++i) {
+        len[i] = clamp_len(p, len[i]);
+        if (PAGED && ub + i < ue && appends(p, len[i]) && (!at || held(at[ub + i]) == len[i]) && !page_ok(p, id[i])) len[i] = -2 - len[i];
+    }
 }
 
 // A CTA's part of the tile sequence.
@@ -100,12 +130,13 @@ struct Share {
 
 // Position in the sequence of tiles: tile j of the stream (unit u, KV head h).  The lengths of units
 // [0, NLEN) sit in shared memory, read once per CTA; those of later units come from the L2.
+template <bool PAGED>
 struct Walker {
     int u, h, j, nt, len;
     bool app;                // the unit's last row is the one this kernel installs
     const int *slen;
     __device__ __forceinline__ void load(const AttnParams &p) {
-        const int raw = u < NLEN ? slen[u] : ld_len(p, u);
+        const int raw = u < NLEN ? slen[u] : ld_len<PAGED>(p, u);
         len = eff_len(p, raw);
         app = appends(p, raw);
         nt = tiles_of(len);
@@ -312,26 +343,35 @@ __device__ __forceinline__ void process_block(uint32_t kt, uint32_t vt, int kb, 
 // The even deal of the tile sequence over the grid, found by all threads of the CTA from len[]: every
 // length is read once (and left in shared memory for units below NLEN), a block-wide prefix sum of tile
 // counts follows, then the two boundaries of this CTA's share.  Boundary c is tile T*c/n_cta; where it
-// falls inside a short stream (<= SNAP tiles) it moves to the nearer end of that stream (finishing a
-// cut stream costs round trips to global memory, more than a few tiles of imbalance); long streams are
-// cut.  sc: [0..5] warp sums, [8] u0, [9] rem, [12] t0, [14] t1.
+// falls inside a short stream (<= SNAP tiles) it moves to the nearer end of that stream, and where it falls
+// within EDGE tiles of an end of a longer one to that end.  Where all units have as many tiles, only as many CTAs
+// take part as share the streams out evenly (ctas_equal).  sc: [0..5] warp sums, [8] u0, [9] rem, [12] t0, [14] t1.
+template <bool PAGED>
 __device__ __forceinline__ Share deal(const AttnParams &p, int *sc, int *slen, int cta) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    auto len_of = [&](int u) { return eff_len(p, u < NLEN ? slen[u] : ld_len(p, u)); };
+    auto len_of = [&](int u) { return eff_len(p, u < NLEN ? slen[u] : ld_len<PAGED>(p, u)); };
     const int per = (p.n_units + THREADS - 1) / THREADS;
     const int ub = min(p.n_units, (int)threadIdx.x * per), ue = min(p.n_units, ub + per);
     int mine = 0;
+    bool same = true;                                             // as many tiles in every unit
     if (per <= LPT) {                                             // all loads in flight together
         int len[LPT];
-        load_lengths(p, ub, ue, len);
+        const int first = ld_len<PAGED>(p, 0);
+        load_lengths<PAGED>(p, ub, ue, len, nullptr);
+        const int nt0 = tiles_of(eff_len(p, first));
 #pragma unroll
         for (int i = 0; i < LPT; ++i)
-            if (ub + i < ue) { slen[ub + i] = len[i]; mine += tiles_of(eff_len(p, len[i])); }
+            if (ub + i < ue) {
+                const int nt = tiles_of(eff_len(p, len[i]));
+                slen[ub + i] = len[i]; mine += nt; same &= nt == nt0;
+            }
     } else {
+        const int nt0 = tiles_of(eff_len(p, ld_len<PAGED>(p, 0)));
         for (int u = ub; u < ue; ++u) {
-            const int len = ld_len(p, u);
+            const int len = ld_len<PAGED>(p, u);
             if (u < NLEN) slen[u] = len;
-            mine += tiles_of(eff_len(p, len));
+            const int nt = tiles_of(eff_len(p, len));
+            mine += nt; same &= nt == nt0;
         }
     }
     int incl = mine;
@@ -341,7 +381,7 @@ __device__ __forceinline__ Share deal(const AttnParams &p, int *sc, int *slen, i
         if (lane >= o) incl += v;
     }
     if (lane == 31) sc[warp] = incl;
-    __syncthreads();
+    same = __syncthreads_and(same);
     int before = 0, all = 0;
 #pragma unroll
     for (int w = 0; w < THREADS / 32; ++w) {
@@ -352,7 +392,7 @@ __device__ __forceinline__ Share deal(const AttnParams &p, int *sc, int *slen, i
     sh.T = (long long)all * p.Hkv;
     // every CTA that takes part owns at least one tile of the even deal, so the CTAs holding a cut stream
     // are consecutive
-    sh.n_cta = (int)min((long long)gridDim.x, sh.T);
+    sh.n_cta = (int)min((long long)(same ? min(p.ctas_equal, (int)gridDim.x) : gridDim.x), sh.T);
     {
         const long long lo = (long long)(before + incl - mine) * p.Hkv, hi = lo + (long long)mine * p.Hkv;
 #pragma unroll
@@ -371,10 +411,8 @@ __device__ __forceinline__ Share deal(const AttnParams &p, int *sc, int *slen, i
                     int rem = (int)(x - pre), uu = u;
                     const int j = rem % nt;
                     long long bx = x;
-                    if (nt <= SNAP && j != 0) {
-                        if (2 * j <= nt) { bx = x - j; rem -= j; }
-                        else { bx = x + (nt - j); rem += nt - j; }
-                    }
+                    if (j != 0 && (nt <= SNAP ? 2 * j <= nt : j <= EDGE)) { bx = x - j; rem -= j; }
+                    else if (j != 0 && (nt <= SNAP || nt - j <= EDGE)) { bx = x + (nt - j); rem += nt - j; }
                     if (rem == nt * p.Hkv) {                      // moved to the start of the next unit that has keys
                         rem = 0;
                         do { ++uu; } while (uu < p.n_units && len_of(uu) == 0);
@@ -397,17 +435,17 @@ __device__ __forceinline__ Share deal(const AttnParams &p, int *sc, int *slen, i
 
 // Address of the first key row of tile w.j of the stream (w.u, w.h) as a row of the cache tensor
 // (contiguous, or through the page table); -1 for a page id out of range.
-__device__ __forceinline__ int tile_row(const AttnParams &p, const Walker &w) {
-    if (!p.page_table) return (w.u * p.Hkv + w.h) * p.cap + w.j * BN;
-    const int row = w.j * BN;
-    const int id = __ldcg(p.page_table + (size_t)w.u * p.pages_per_unit + row / p.page_rows);
-    if (id < 0 || id >= p.n_pages) return -1;
+template <bool PAGED>
+__device__ __forceinline__ int tile_row(const AttnParams &p, const Walker<PAGED> &w) {
+    if (!PAGED) return (w.u * p.Hkv + w.h) * p.cap + w.j * BN;
+    const int row = w.j * BN, id = ld_page(p, w.u, row);
+    if (!page_ok(p, id)) return -1;
     return (id * p.Hkv + w.h) * p.page_rows + row % p.page_rows;
 }
 
 // GP: the group size G rounded up to a power of two (1 .. 16); it fixes how the finishing warp's lanes
 // map to (query head, features) and how many n-tiles of 8 heads the MMAs span.
-template <int DH, int GP>
+template <int DH, int GP, bool PAGED>
 __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
 coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                    const __grid_constant__ CUtensorMap tm_k_end, const __grid_constant__ CUtensorMap tm_v_end) {
@@ -428,6 +466,7 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
     int *sc = reinterpret_cast<int *>(tail + 128);              // scalars of the deal, [11] dead,
     volatile int *dead = sc + 11;                               // [16..23] description of the stream in `red`
     volatile int *meta = sc + 16;
+    volatile int *tile_at = sc + 24;                            // [STAGES] first cache row of the tile in a stage
     int *slen = sc + 32;                                        // [NLEN] lengths of the first units
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -457,10 +496,10 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
     // Batches beyond NLEN units keep no copy to compare with and deal after the wait.
     const bool ahead = p.n_units <= NLEN;
     Share sh;
-    Walker w;
+    Walker<PAGED> w;
     bool started = false;
     if (ahead) {
-        sh = deal(p, sc, slen, cta);
+        sh = deal<PAGED>(p, sc, slen, cta);
         if (sh.t0 < sh.t1) started = w.start(p, sh, slen);
     }
 
@@ -468,11 +507,10 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
     // there and the row a folded-in append installs if the stream ends there.  whole_box: fetch a box of BN
     // rows whatever the length says (for loads that go out before the lengths are confirmed: a unit may have
     // grown inside its last tile since they were read; what lies past the end of a cache is never used).
-    auto issue_tile = [&](int it, const Walker &tw, bool whole_box) {
+    // y: row of the tile's first key in the cache tensor.
+    auto issue_tile = [&](int it, const Walker<PAGED> &tw, int y, bool whole_box) {
         const int s = it % STAGES;
-        // row of the tile's first key in the cache tensor; for a paged cache through the page table
-        int y = tile_row(p, tw);
-        if (y < 0) { atomicOr(p.status, PHOTON_DEV_BAD_INDEX); y = tw.h * (p.page_table ? p.page_rows : p.cap); }
+        if (PAGED && y < 0) { atomicOr(p.status, PHOTON_DEV_BAD_INDEX); y = tw.h * p.page_rows; }
         const uint32_t full = bars + 16 * s;
         const uint32_t kd = base + s * R::STAGE_BYTES, vd = kd + R::TILE_BYTES;
         const int rows = min(BN, tw.len - tw.j * BN);
@@ -480,6 +518,7 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
         // a tile of more than BOX rows comes as one box of BN rows per 64 features, a shorter one as one box of BOX rows
         const bool tall = whole_box || rows > BOX;
         const bool grows = tw.app && tw.j == tw.nt - 1;        // the row this kernel installs lies in this tile
+        if (PAGED) tile_at[s] = y;
         ptx::mbar_arrive_expect_tx(full, R::HALVES * (tall ? HALF_BYTES : BOX_BYTES) * 2 + (first ? G * DH * 2 : 0) +
                                              (grows ? NB : 0));
 #pragma unroll
@@ -503,9 +542,23 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
     // values and queries are final now, only the deal may turn out stale.  If it does (rare), these loads are
     // left to land, the ring's barriers are made anew and everything starts over from the deal.
     int n_early = 0;
-    if (ahead && started && warp == NW && lane == 0) {
+    if (ahead && started && warp == NW) {
         const int n = (int)min((long long)STAGES, sh.t1 - sh.t0);
-        for (; n_early < n && w.valid(p); ++n_early, w.next(p)) issue_tile(n_early, w, !p.k_new);
+        if (PAGED) {                        // the page ids of these tiles in one trip, a lane each
+            Walker<PAGED> lw = w;
+            for (int i = 0; i < lane && i < n && lw.valid(p); ++i) lw.next(p);
+            const int y_lane = lane < n && lw.valid(p) ? tile_row(p, lw) : 0;
+            __syncwarp();
+#pragma unroll 1
+            for (int i = 0; i < n && w.valid(p); ++i) {
+                const int y = __shfl_sync(0xffffffffu, y_lane, i);
+                if (lane == 0) issue_tile(i, w, y, !p.k_new);
+                n_early = i + 1;
+                w.next(p);
+            }
+        } else if (lane == 0) {
+            for (; n_early < n && w.valid(p); ++n_early, w.next(p)) issue_tile(n_early, w, tile_row(p, w), !p.k_new);
+        }
     }
 
     bool redo = !ahead;
@@ -513,7 +566,7 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
         const int per = (p.n_units + THREADS - 1) / THREADS;
         const int ub = min(p.n_units, (int)threadIdx.x * per), ue = min(p.n_units, ub + per);
         int diff = 0, len[LPT];
-        load_lengths(p, ub, ue, len);
+        load_lengths<PAGED>(p, ub, ue, len, slen);
 #pragma unroll
         for (int i = 0; i < LPT; ++i)
             if (ub + i < ue) {
@@ -540,7 +593,7 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
             }
         }
         if (threadIdx.x == 0) { sc[8] = -1; sc[9] = 0; sc[12] = 0; sc[14] = -1; }
-        sh = deal(p, sc, slen, cta);
+        sh = deal<PAGED>(p, sc, slen, cta);
         started = sh.t0 < sh.t1 && w.start(p, sh, slen);
     } else if (started && w.valid(p)) {
         w.load(p);                          // same tile counts, but the unit may have grown within its last tile
@@ -559,13 +612,13 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
             if (last) *p.readers = 0;                          // zero again for the next call
         }
         if (__shfl_sync(0xffffffffu, last, 0)) {
-            bool full = false;
+            int bits = 0;
             for (int u = lane; u < p.n_units; u += 32) {
                 const int raw = slen[u];
                 if (appends(p, raw)) p.len_w[u] = raw + 1;
-                else full = true;
+                else bits |= PAGED && raw <= -2 ? PHOTON_DEV_BAD_INDEX : PHOTON_DEV_CAPACITY;
             }
-            if (full) atomicOr(p.status, PHOTON_DEV_CAPACITY);
+            if (bits) atomicOr(p.status, bits);
         }
     }
 
@@ -573,7 +626,7 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
     // (the whole CTA when it has no tiles, else the finishing warp before its first stream arrives)
     auto finish_empty_units = [&](int tid, int nthreads) {
         for (int u = cta; u < p.n_units; u += gridDim.x) {
-            if (eff_len(p, u < NLEN ? slen[u] : ld_len(p, u)) != 0) continue;
+            if (eff_len(p, u < NLEN ? slen[u] : ld_len<PAGED>(p, u)) != 0) continue;
             for (int idx = tid; idx < p.Hq * DH; idx += nthreads)
                 emit<DH>(p, u, idx / DH, idx % DH, 0.f, -CUDART_INF_F, 0.f);
         }
@@ -599,7 +652,7 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
         const bool row_ok = r < G, lead = row_ok && (lane % lpr == 0);
         finish_empty_units(lane, 32);
         // it walks the streams of this CTA in the consumers' order, one step ahead of them
-        Walker fw = w;
+        Walker<PAGED> fw = w;
         for (int sidx = 0;; ++sidx) {
             SharedPart<MAXV> sp;
             sp.sid = -1;
@@ -720,11 +773,12 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
                 if (!w.valid(p)) {                               // ran past the last unit: len[] changed under the kernel
                     *dead = 1; atomicOr(p.status, PHOTON_DEV_BAD_INDEX); break;
                 }
+                const int y = tile_row(p, w);                    // (a page id is on its way while the stage is waited for)
                 // the ring starts empty: only from its second turn on is there a stage to wait for
                 if (it >= STAGES && !ptx::mbar_wait(bars + 16 * s + 8, ((it / STAGES) & 1) ^ 1)) {
                     *dead = 1; atomicOr(p.status, PHOTON_DEV_TIMEOUT); break;
                 }
-                issue_tile(it, w, false);
+                issue_tile(it, w, y, false);
             }
             if (*dead) {
                 // loads already issued still land in this CTA's shared memory: give them time to finish
@@ -788,7 +842,7 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
                     const uint4 piece = ptx::lds128(n_base + s * NB + lane * 16);
                     const uint32_t tile = base + s * R::STAGE_BYTES + (is_v ? R::TILE_BYTES : 0);
                     ptx::sts128(tile + (cf >> 3) * HALF_BYTES + r * 128 + (((cf & 7) ^ (r & 7)) << 4), piece);
-                    const size_t row = ((size_t)w.u * p.Hkv + w.h) * p.cap + (w.len - 1);
+                    const size_t row = PAGED ? (size_t)tile_at[s] + r : ((size_t)w.u * p.Hkv + w.h) * p.cap + (w.len - 1);
                     *reinterpret_cast<uint4 *>((is_v ? p.v_w : p.k_w) + row * DH + cf * 8) = piece;
                 }
                 __syncwarp();
@@ -842,8 +896,8 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
                 if (!whole) {
                     // CTAs that hold a piece of this stream: first and last
                     const long long te = seg_t + w.nt;
-                    meta[3] = (int)(((seg_t + 1) * n_cta - 1) / T);
-                    meta[4] = (int)((te * n_cta - 1) / T);
+                    meta[3] = (int)(((seg_t + EDGE + 1) * n_cta - 1) / T);     // (boundaries within EDGE tiles of an end have moved there)
+                    meta[4] = (int)(((te - EDGE) * n_cta - 1) / T);
                 }
             }
             if (direct) ptx::named_bar_sync(1, NW * 32);
@@ -886,12 +940,12 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
     }
 }
 
-template <int DH, int GP>
+template <int DH, int GP, bool PAGED>
 cudaError_t run(photon_ctx *ctx, AttnParams p, cudaStream_t st, long long *launches) {
     const int G = p.Hq / p.Hkv;
     const size_t smem = smem_bytes<DH>(G);
     static size_t smem_set[kMaxDevices] = {};
-    if (const cudaError_t e = ensure_dynamic_smem(coarse_attn_kernel<DH, GP>, smem, ctx->device, smem_set)) return e;
+    if (const cudaError_t e = ensure_dynamic_smem(coarse_attn_kernel<DH, GP, PAGED>, smem, ctx->device, smem_set)) return e;
     const CUtensorMap *t;
     CUtensorMap mk, mv, mk_end, mv_end;
     const uint64_t pool_rows = p.page_table ? (uint64_t)p.n_pages * p.Hkv * p.page_rows : (uint64_t)p.n_units * p.Hkv * p.cap;
@@ -905,9 +959,14 @@ cudaError_t run(photon_ctx *ctx, AttnParams p, cudaStream_t st, long long *launc
     mv_end = *t;
     const int max_len = p.k_new ? std::min(p.max_len + 1, p.cap) : p.max_len;     // a folded-in append grows every unit by a row
     const long long t_max = (long long)p.n_units * p.Hkv * ((max_len + BN - 1) / BN);
-    const long long cap = ctx->attn_ctas > 0 ? ctx->attn_ctas : coarse_attn_grid(ctx->max_ctas, (long long)p.n_units * p.Hkv);
+    const long long streams = (long long)p.n_units * p.Hkv;
+    p.ctas_equal = ctx->attn_ctas > 0 ? ctx->attn_ctas : coarse_attn_grid(ctx->max_ctas, streams);
+    // More streams than that: which CTAs take part is decided on the device, by whether the lengths are equal.  (Not with very many
+    // streams: they even out by themselves, and the CTAs that leave at once cost a step of 512 x 8 streams 2.7 of 241 us.)
+    const bool by_lengths = ctx->attn_ctas <= 0 && streams > p.ctas_equal && streams <= 8ll * ctx->max_ctas;
+    const long long cap = by_lengths ? ctx->max_ctas : p.ctas_equal;
     const int grid = (int)std::max<long long>(1, std::min<long long>(t_max, cap));
-    const cudaError_t e = launch_dependent(coarse_attn_kernel<DH, GP>, dim3(grid), dim3(THREADS), smem, st, 0, p, mk, mv, mk_end, mv_end);
+    const cudaError_t e = launch_dependent(coarse_attn_kernel<DH, GP, PAGED>, dim3(grid), dim3(THREADS), smem, st, 0, p, mk, mv, mk_end, mv_end);
     ++*launches;
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -917,26 +976,23 @@ cudaError_t run(photon_ctx *ctx, AttnParams p, cudaStream_t st, long long *launc
 int coarse_attn_ctas_per_sm() { return CTAS_PER_SM; }
 int coarse_attn_fold_limit() { return NLEN; }
 
-// The grid when the caller sets none.  Not every CTA slot of the device is taken: the kernel is bound by
-// HBM well below that, and a slot left free lets a CTA of the next kernel in the stream start, and get
+// The CTAs that share the work when all units have as many tiles.  Not every CTA slot of the device is taken: the kernel is
+// bound by HBM well below that, and a slot left free lets a CTA of the next kernel in the stream start, and get
 // through its set-up, while this one still runs (measured on caches of 64 to 256 MiB: 7/8 of the slots is 1 to 4 %
-// faster than all of them).  Below that bound the grid is a multiple or a near-divisor of the number of
-// (unit, KV head) streams, so that in a batch of equal lengths every stream falls to the same whole
-// number of CTAs, or every CTA to the same whole number of streams, and the cuts of the even deal line
-// up with the streams' ends; with ragged lengths the deal is even whatever the grid.
+// faster than all of them).  Up to that many (unit, KV head) streams the grid is a multiple of their number, so that every
+// stream falls to the same whole number of CTAs and the cuts of the deal line up with the streams' ends; with more it is what
+// makes as few rounds of whole streams as there can be, the last eighth of the slots included where that saves more than its
+// share (200 sequences of 150 rows, 4 KV heads: 16.4 -> 15.3 us with 267 CTAs
+// instead of 200; 130 of 1000: 48.9 -> 45.4).  Where lengths differ all slots are taken then: the more CTAs, the more of them are left
+// to share the bandwidth of those that are through (77 sequences of 0 to 1000 rows: 195 CTAs 22.4 us, 259 19.2, 296 18.6).
 int coarse_attn_grid(int resident_ctas, long long n_streams) {
     const int top = std::max(1, resident_ctas * 7 / 8);
     if (n_streams <= 0) return 1;
     if (n_streams <= top) return (int)(n_streams * (top / n_streams));
-    // more streams than CTAs: the grid within the upper quarter that wastes the fewest stream slots
-    int best = top;
-    long long best_waste = -1;
-    for (int g = top; g >= top - top / 4; --g) {
-        const long long waste = (n_streams + g - 1) / g * g - n_streams;
-        if (best_waste < 0 || waste < best_waste) { best = g; best_waste = waste; }
-        if (waste == 0) break;
-    }
-    return best;
+    // more streams than CTAs: as few whole streams per CTA as there can be, and no more CTAs than that takes
+    const long long rounds = (n_streams + top - 1) / top, fewest = (n_streams + resident_ctas - 1) / resident_ctas;
+    const long long r = fewest * 8 < rounds * 7 ? fewest : rounds;
+    return (int)std::max<long long>(top - top / 4, (n_streams + r - 1) / r);
 }
 
 cudaError_t launch_attention(photon_ctx *ctx, const AttnParams &p, cudaStream_t st, long long *launches) {
@@ -952,7 +1008,8 @@ cudaError_t launch_attention(photon_ctx *ctx, const AttnParams &p, cudaStream_t 
     const int G = p.Hq / p.Hkv;
     int gp = 1;
     while (gp < G) gp <<= 1;
-#define PHOTON_COARSE_CASE(D, GPV) if (p.dh == D && gp == GPV) return run<D, GPV>(ctx, p, st, launches);
+#define PHOTON_COARSE_CASE(D, GPV) if (p.dh == D && gp == GPV) \
+        return p.page_table ? run<D, GPV, true>(ctx, p, st, launches) : run<D, GPV, false>(ctx, p, st, launches);
     PHOTON_COARSE_CASE(128, 1) PHOTON_COARSE_CASE(128, 2) PHOTON_COARSE_CASE(128, 4) PHOTON_COARSE_CASE(128, 8)
     PHOTON_COARSE_CASE(128, 16)
     PHOTON_COARSE_CASE(64, 1) PHOTON_COARSE_CASE(64, 2) PHOTON_COARSE_CASE(64, 4) PHOTON_COARSE_CASE(64, 8)

@@ -73,6 +73,7 @@ struct AttnParams {
     const int32_t *page_table;   // paged cache: [n_units, pages_per_unit] page ids, or NULL
     int page_rows, pages_per_unit, n_pages;
     int n_q, Hq, Hkv, dh;
+    int ctas_equal;          // filled by the launcher: CTAs of the coarse attention that take part when every unit has as many tiles
     int splits_sh;           // key ranges of a shared prefix = cluster size of its kernel (0: no shared prefix)
     int upc;                 // filled by the launcher: units per CTA on shared keys
     int own_rows;            // filled by the launcher: the units' own keys (at most this many rows each) are read by the
@@ -85,7 +86,7 @@ struct AttnParams {
     int32_t *tickets;
     int32_t *status;
     // The step's append folded into the attention over the unit's own keys (all NULL otherwise): one new row per unit,
-    // k_new, v_new [n_units, Hkv, dh], installed at row len[u] of a contiguous cache (k_w, v_w: the cache, writable),
+    // k_new, v_new [n_units, Hkv, dh], installed at row len[u] of the unit's cache (k_w, v_w: the cache or the pools, writable),
     // len_w[u] += 1 by the last CTA to arrive on `readers` (a counter that is zero between calls).
     const bf16 *k_new, *v_new;
     bf16 *k_w, *v_w;

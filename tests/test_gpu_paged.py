@@ -118,3 +118,77 @@ def test_bad_pages_and_calls_that_do_not_take_pages():
         kv.page_rows = 48                                                 # not a multiple of 64
         with pytest.raises(ph.PhotonError):
             ph.photon_coarse_attn(c.h, kv, q, out, None, 1.0)
+
+
+@pytest.mark.parametrize("Hq,Hkv,dh", [(16, 4, 128), (8, 8, 128), (4, 2, 64)])
+def test_step_on_pages_appends_inside_the_attention(Hq, Hkv, dh):
+    """The step folds the append into the attention for paged caches too: against append and attention called one after the
+    other, same bits, same cache, lengths and status.  Units that are empty, one row short of a page, at a page's first row,
+    full, and one whose next page does not exist."""
+    cfg = wl.scaled(wl.CONFIGS[1], B=9, Hq=Hq, Hkv=Hkv, dh=dh, D=Hq * dh)
+    B, page_rows, ppu, P = 9, 128, 3, cfg.P
+    n_pages, cap, scale = B * ppu, 384, dh ** -0.5
+    g = torch.Generator("cuda").manual_seed(Hq)
+
+    def rand(*shape, std=1.0):
+        return (torch.randn(*shape, generator=g, device="cuda") * std).to(torch.bfloat16)
+
+    lens = np.array([0, 63, 64, 127, 128, 200, cap, 255, 256], np.int32)
+    table = np.random.default_rng(3).permutation(n_pages).reshape(B, ppu).astype(np.int32)
+    table[8, 2] = n_pages                                                # unit 8 is at the first row of a page that is not there
+    table_dev, pk, pv = dev_i32(table), rand(n_pages, Hkv, page_rows, dh), rand(n_pages, Hkv, page_rows, dh)
+    k_new, v_new, q, w = rand(B, Hkv, dh), rand(B, Hkv, dh), rand(B, Hq, dh), rand(Hq * dh, P * Hq * dh, std=0.02)
+    got = []
+    with Ctx(cfg) as c:
+        for folded in (False, True):
+            k, v, ln = pk.clone(), pv.clone(), dev_i32(lens)
+            kv = ph.make_kv(k, v, ln, page_table=table_dev)
+            out, lse = torch.empty_like(q), torch.empty(B, Hq, device="cuda")
+            n0 = ph.photon_launch_count(c.h)
+            if folded:
+                U = torch.empty(B, P, Hq * dh, dtype=torch.bfloat16, device="cuda")
+                args = ph.make_step_args(kv, k_new, v_new, q, out, scale, w, ph.PHOTON_W_IN_MAJOR, U, B, lse_coarse=lse)
+                ph.photon_decode_step(c.h, args)
+                assert ph.photon_launch_count(c.h) - n0 == 2
+            else:
+                ph.photon_kv_append(c.h, kv, k_new, v_new)
+                ph.photon_coarse_attn(c.h, kv, q, out, lse, scale)
+            assert c.status() == ph.PHOTON_DEV_CAPACITY | ph.PHOTON_DEV_BAD_INDEX
+            got.append([host_bits(t) for t in (out, k, v)] + [lse.cpu().numpy(), ln.cpu().numpy()])
+    assert np.array_equal(got[0][-1], lens + np.array([1, 1, 1, 1, 1, 1, 0, 1, 0]))
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n,S,lengths", [(80, 1100, "ragged"), (80, 1024, "equal"), (75, 1088, "equal"), (3, 3000, "ragged"), (300, 70, "ragged"),
+                                         (20, 1300, "one long"), (70, 2200, "ragged")])
+@pytest.mark.parametrize("paged", [False, True])
+def test_streams_at_the_edges_of_the_deal(n, S, lengths, paged):
+    """More streams than CTAs, lengths equal (fewer CTAs take part) and not, streams of 16 tiles (never cut) and of 17 (cut, but not
+    close to their ends).  Against torch in 64 bits: half a bf16 step of values below 4 (2^-7), and the weights' rounding."""
+    Hq, Hkv, dh = 8, 4, 64
+    cfg = wl.scaled(wl.CONFIGS[1], B=n, Hq=Hq, Hkv=Hkv, dh=dh, D=Hq * dh)
+    rng = np.random.default_rng(n)
+    lens = (np.full(n, S) if lengths == "equal" else rng.integers(0, S + 1, n) if lengths == "ragged" else np.where(np.arange(n) == 7, S, 40)).astype(np.int32)
+    g = torch.Generator("cuda").manual_seed(n)
+    k, v, q = ((torch.randn(*s, generator=g, device="cuda")).to(torch.bfloat16) for s in ((n, Hkv, S, dh), (n, Hkv, S, dh), (n, Hq, dh)))
+    out, lse = torch.empty_like(q), torch.empty(n, Hq, device="cuda")
+    with Ctx(cfg) as c:
+        if paged:
+            ppu = -(-S // 64)
+            pad = lambda t: torch.nn.functional.pad(t, (0, 0, 0, ppu * 64 - S)).view(n, Hkv, ppu, 64, dh).transpose(1, 2).reshape(n * ppu, Hkv, 64, dh)
+            order = torch.randperm(n * ppu, generator=g, device="cuda")
+            pk, pv = torch.empty_like(pad(k)), torch.empty_like(pad(v))
+            pk[order], pv[order] = pad(k), pad(v)
+            kv = ph.make_kv(pk, pv, dev_i32(lens), page_table=order.to(torch.int32).view(n, ppu).contiguous())
+        else:
+            kv = ph.make_kv(k, v, dev_i32(lens))
+        ph.photon_coarse_attn(c.h, kv, q, out, lse, dh ** -0.5)
+        assert c.status() == 0
+    logit = torch.einsum("nhgd,nhsd->nhgs", q.double().view(n, Hkv, Hq // Hkv, dh), k.double()) * dh ** -0.5
+    logit.masked_fill_((torch.arange(S, device="cuda") >= torch.from_numpy(lens).cuda()[:, None])[:, None, None], float("-inf"))
+    want = torch.einsum("nhgs,nhsd->nhgd", torch.softmax(logit, -1).nan_to_num(0.0), v.double()).reshape(n, Hq, dh)
+    assert (out.double() - want).abs().max() <= 2e-2
+    want_lse = torch.logsumexp(logit, -1).view(n, Hq)
+    fin = torch.isfinite(want_lse)
+    assert torch.equal(torch.isneginf(lse), ~fin) and (lse.double() - want_lse)[fin].abs().max() < 2e-3
