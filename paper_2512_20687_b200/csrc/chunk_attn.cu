@@ -477,14 +477,11 @@ cudaError_t launch(photon_ctx *ctx, const AttnParams &p, cudaStream_t st, long l
     //  - with fewer heads at a time, or longer buffers: there the compiler gives the small CTA too few registers and its row loads
     //    wait for one another (8/8 x 128, 24 rows: 128 chunks 4.2 / 9.0; 16/4 x 128, 48 rows: 1000 chunks 37 / 57);
     //  - of 24 rows, up to one wave of eight-warp CTAs (16/4 x 128: 256 chunks 5.8 / 7.7; beyond it about equal);
-    //  - beside the coarse part of a captured step, up to one wave: there the two start together, and spread over all SMs the small
-    //    CTAs are in the way of the coarse attention's second CTA per SM (step of 64 sequences with 2 chunks each, replayed: 28.1 /
-    //    29.6 us; launched one by one the chunk attention is ahead, and the small CTAs leave the SMs sooner: 31.7 / 30.1);
     //  - where queries and results cross the bus: hundreds of resident CTAs that wait for it (280 sequences with 8 chunks each,
     //    host-driven: 330 / 350; 64 with 2: 57.4 / 63.0).
     if constexpr (GT == 4 && RP <= 24) {
         const bool one_wave = items <= (long long)CH_WARPS * ctx->sm_count;
-        if (!p.over_bus && !(one_wave && (p.replayed_beside || RP == 24))) {
+        if (!p.over_bus && !(one_wave && RP == 24)) {
             chunk_attn_kernel<DH, RP, GT, 1><<<(unsigned)items, 32, 0, st>>>(p);
             ++*launches;
             return cudaGetLastError();

@@ -78,8 +78,7 @@ struct AttnParams {
     int upc;                 // filled by the launcher: units per CTA on shared keys
     int own_rows;            // filled by the launcher: the units' own keys (at most this many rows each) are read by the
                              // shared-prefix kernel, which then writes the final result; 0: a second kernel reads them
-    // chunk attention: beside the coarse part of a step that is being captured; queries and results in host memory
-    bool replayed_beside, over_bus;
+    bool over_bus;           // chunk attention: queries and results in host memory
     float scale_log2;        // scale * log2(e): logits are kept in the base-2 domain
     float *partials;
     float *cta_partials;

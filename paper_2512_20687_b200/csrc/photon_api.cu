@@ -39,7 +39,7 @@ int ceil_div(int a, int b) { return (a + b - 1) / b; }
 photon_status attention_common(photon_ctx *ctx, const photon_kv *cache, const photon_bf16 *q,
                                const int32_t *slot, int n_q, photon_bf16 *out, float *lse,
                                float scale, bool chunk, cudaStream_t st, const photon_bf16 *k_new = nullptr,
-                               const photon_bf16 *v_new = nullptr, bool replayed_beside = false, bool over_bus = false) {
+                               const photon_bf16 *v_new = nullptr, bool over_bus = false) {
     if (!ctx) return PHOTON_ERR_INVALID_ARG;
     if (!kv_ok(ctx, cache, !chunk) || (chunk && cache->page_table)) return PHOTON_ERR_INVALID_ARG;
     if (n_q < 0 || (n_q > 0 && (!q || !out))) return PHOTON_ERR_INVALID_ARG;
@@ -81,7 +81,6 @@ photon_status attention_common(photon_ctx *ctx, const photon_kv *cache, const ph
         p.len_w = cache->len;
         p.readers = ctx->readers;
     }
-    p.replayed_beside = replayed_beside;
     p.over_bus = over_bus;
     p.max_len = cache->max_len ? cache->max_len : cache->cap;
     p.splits_sh = 0;
@@ -604,16 +603,25 @@ photon_status step_impl(photon_ctx *ctx, const photon_step_args *a, photon_strea
         if (!forked && (cudaEventRecord(ctx->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0) != cudaSuccess))
             return PHOTON_ERR_CUDA;
         if (apart && !direct && !copy_in(hp, hp->in_split, hp->in_bytes, ctx->side)) s = PHOTON_ERR_CUDA;
-        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) s = PHOTON_ERR_CUDA;
+    }
+    // every way out from here on joins the side stream again, failed calls included
+    auto chunks_beside = [&]() {
         if (s == PHOTON_OK)
             s = attention_common(ctx, a->chunks, q_chunk, slot, a->Nc, out_chunk, nullptr, a->scale_chunk, true, ctx->side, nullptr,
-                                 nullptr, capture != cudaStreamCaptureStatusNone, direct);
+                                 nullptr, direct);
         if (s == PHOTON_OK && apart && !direct && !copy_out(hp, hp->out_split, hp->out_bytes, ctx->side)) s = PHOTON_ERR_CUDA;
-        // every way out from here on joins the side stream again, failed calls included
-        if (cudaEventRecord(ctx->ev_join, ctx->side) != cudaSuccess) s = PHOTON_ERR_CUDA;
-        if (s != PHOTON_OK) { cudaStreamWaitEvent(st, ctx->ev_join, 0); return s; }
-    }
+        if (cudaEventRecord(ctx->ev_join, ctx->side) != cudaSuccess && s == PHOTON_OK) s = PHOTON_ERR_CUDA;
+        if (s != PHOTON_OK) cudaStreamWaitEvent(st, ctx->ev_join, 0);
+        return s;
+    };
+    // Called one by one the chunk attention goes to its stream first: it is launched while the coarse part's kernel is still on its
+    // way.  In a captured step both start at the same time, and where the chunk attention is the first node its CTAs take
+    // registers from the coarse attention's first wave: there it follows (replayed, 64 sequences 25.2 -> 23.6 us, 16 long ones
+    // 60.1 -> 57.9, 77 ragged paged ones 40.3 -> 37.0; called one by one that order is no faster, the long ones 59.8 and 60.5).
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (beside && cudaStreamIsCapturing(st, &capture) != cudaSuccess) s = PHOTON_ERR_CUDA;
+    const bool chunks_first = capture == cudaStreamCaptureStatusNone;
+    if (beside && (chunks_first || s != PHOTON_OK) && chunks_beside() != PHOTON_OK) return s;
     // The append is one row per unit, in place: for a batch whose lengths fit the attention kernel's shared memory it
     // is folded into that kernel (the warp that reaches a unit's last tile installs the
     // new row in the tile and in the cache; the lengths grow once every CTA has read them), which takes a launch
@@ -629,6 +637,7 @@ photon_status step_impl(photon_ctx *ctx, const photon_step_args *a, photon_strea
                  : photon_coarse_attn(ctx, a->coarse, a->q_coarse, a->out_coarse, a->lse_coarse, a->scale_coarse, stream);
     if (s == PHOTON_OK && a->ev_attn_end && cudaEventRecord(static_cast<cudaEvent_t>(a->ev_attn_end), st) != cudaSuccess)
         s = PHOTON_ERR_CUDA;
+    if (beside && !chunks_first && chunks_beside() != PHOTON_OK) return s;
     // What the coarse attention wrote leaves beside the converter.  Where the converter's own output lies in the
     // coarse part of the staging area, it and whatever follows it there leave after the converter.
     size_t early_end = hp ? hp->out_split : 0;
@@ -650,7 +659,7 @@ photon_status step_impl(photon_ctx *ctx, const photon_step_args *a, photon_strea
         if (cudaStreamWaitEvent(st, ctx->ev_join, 0) != cudaSuccess && s == PHOTON_OK) s = PHOTON_ERR_CUDA;
     } else if (s == PHOTON_OK && a->Nc > 0) {
         s = attention_common(ctx, a->chunks, q_chunk, slot, a->Nc, out_chunk, nullptr, a->scale_chunk, true, st, nullptr, nullptr,
-                             false, direct);
+                             direct);
     }
     if (copying && cudaStreamWaitEvent(st, ctx->ev_copy, 0) != cudaSuccess && s == PHOTON_OK) s = PHOTON_ERR_CUDA;
     if (s == PHOTON_OK && hp && !copy_out(hp, copying ? early_end : 0, apart || direct ? hp->out_split : hp->out_bytes, st))
