@@ -231,7 +231,9 @@ photon_status photon_linear(photon_ctx *ctx, const photon_bf16 *x, const photon_
  * the newest in-chunk position of every in-flight chunk: `chunks` holds the
  * chunk buffers (cap <= P + C; x, y [n_units, D]), the position is the
  * buffer's length before the append (prefix rows count), and the attention
- * is the bounded one of photon_chunk_attn.
+ * is the bounded one of photon_chunk_attn.  With many chunks the projection's
+ * own epilogue rotates, splits and appends (rounding to bf16 first, as when the
+ * projection is stored and read back), and scratch->qkv is left unwritten.
  *
  * photon_decoder_prefill: the same layer over a fresh converter prefix, the
  * first R_l positions of the sequence [U ; X_<j] of Eq. 6: U [n, P, D] (what
@@ -251,7 +253,7 @@ typedef struct photon_layer {
 } photon_layer;
 typedef struct photon_layer_scratch {
   photon_bf16 *n;            /* [B, D]   normalised input of either half */
-  photon_bf16 *qkv;          /* [B, (Hq + 2 Hkv) dh] */
+  photon_bf16 *qkv;          /* [B, (Hq + 2 Hkv) dh]  unwritten by photon_decoder_step with many chunks */
   photon_bf16 *q;            /* [B, Hq, dh] */
   photon_bf16 *k_new, *v_new;/* [B, Hkv, dh]  written by photon_decoder_prefill only */
   photon_bf16 *att;          /* [B, Hq, dh] */

@@ -92,6 +92,8 @@ chunk_causal_attn_kernel(const CausalParams p) {
     using S = Shape<DH, KT>;
     constexpr int ROWB = S::ROWB, CPR = S::CPR, RPI = S::RPI, NC = S::NC;
     extern __shared__ __align__(128) uint8_t smem[];
+    ptx::grid_dep_wait();                   // (one wave of CTAs: only the launch itself runs under the kernel before this one)
+    ptx::grid_dep_launch();
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_warps = blockDim.x >> 5;
@@ -177,6 +179,10 @@ chunk_causal_attn_kernel(const CausalParams p) {
         const bool bad = it.u < 0 || it.u >= p.n_units;
         if (bad && lane == 0) atomicOr(p.status, PHOTON_DEV_BAD_INDEX);
         it.len = bad ? 0 : max(0, min(__ldcg(p.len + it.u), p.cap));
+        if (p.grown && !bad) {
+            const int n = __ldcg(p.len + it.u);
+            if (n >= 0 && n + p.grown <= p.cap) it.len = n + p.grown;
+        }
         it.n_keys = p.row0 < it.len ? min(it.len, p.row0 + p.R) : 0;   // rows any query of this call can see
         it.kt_all = (it.n_keys + 15) >> 4;
         return it;
@@ -403,9 +409,9 @@ cudaError_t launch(photon_ctx *ctx, CausalParams p, cudaStream_t st, long long *
     const unsigned grid = (unsigned)std::min<long long>(ctx->sm_count, (items + w - 1) / w);
     cudaError_t e = ensure_dynamic_smem(chunk_causal_attn_kernel<DH, KT>, (size_t)W * S::WARP_BYTES, ctx->device, attr_set);
     if (e != cudaSuccess) return e;
-    chunk_causal_attn_kernel<DH, KT><<<grid, w * 32, (size_t)w * S::WARP_BYTES, st>>>(p);
+    e = launch_dependent(chunk_causal_attn_kernel<DH, KT>, dim3(grid), dim3(w * 32), (size_t)w * S::WARP_BYTES, st, 0, p);
     ++*launches;
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int DH>

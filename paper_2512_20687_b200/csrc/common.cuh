@@ -96,6 +96,7 @@ struct AttnParams {
 // Whole-chunk causal attention: query t of item i (q, out: [n, R, Hq, dh]) stands at row row0 + t of
 // chunk buffer u = slot ? slot[i] : i and sees rows 0 .. row0 + t of it.
 struct CausalParams {
+    int grown;               // rows that every unit with room for them has been given beyond len (len itself grows later)
     const bf16 *q;
     bf16 *out;
     const bf16 *k, *v;
@@ -108,6 +109,18 @@ struct CausalParams {
     int Hq, Hkv, dh;
     float scale_log2;
     int32_t *status;
+};
+
+// What becomes of a fused q/k/v projection in its own epilogue (q == NULL: nothing): rows [.., (Hq + 2 Hkv) dh] are taken apart,
+// q and k rotated (half-split pairing, base 2^log2_theta), and k and v written into a contiguous cache.
+// period 0: row i is unit i, at the position of its length.  period P: rows of P positions 0 .. P-1 each, item i / P goes to unit
+// unit_ids[i / P] (or i / P), at row len + i % P; k_new and v_new get a copy.  A unit without room for all its rows gets none.
+struct RopeOut {
+    bf16 *q, *k_new, *v_new, *k_cache, *v_cache;
+    bf16 *qkv;               // the projection as it is, or NULL
+    const int32_t *len, *unit_ids;
+    int n_units, cap, period, Hq, Hkv, dh;
+    double log2_theta;
 };
 
 struct ConvParams {
@@ -126,6 +139,7 @@ struct ConvParams {
     int stages;              // filled by the launcher: stages of the ring
     int once;                // filled by the launcher: weights ahead, and no slice of K is longer than the ring
     int32_t *status;
+    RopeOut rope;
 };
 
 // Raises a kernel's dynamic shared-memory limit once per device (the attribute is per device and per
@@ -194,6 +208,17 @@ cudaError_t launch_chunk_attention(photon_ctx *ctx, const AttnParams &p, cudaStr
                                    long long *launches);
 cudaError_t launch_chunk_causal_attention(photon_ctx *ctx, const CausalParams &p, cudaStream_t st,
                                           long long *launches);
+// a fused q/k/v projection (p.rope.q set), by either kernel
+cudaError_t launch_qkv_rope(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches);
+cudaError_t launch_qkv_rope_pairs(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches);
+// len of the units that such a projection of n items has given rows to grows by n_rows each, with the append kernel's checks
+struct Grow {
+    int32_t *len;
+    const int32_t *unit_ids;
+    int n_units, cap, n, n_rows;
+    int32_t *status;
+};
+cudaError_t launch_grow(const Grow &g, cudaStream_t st, long long *launches);
 cudaError_t launch_linear(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches);
 cudaError_t linear_cluster_counts(int device, int (&fit)[MAX_CLUSTER + 1]);
 // for tests: {columns per tile, CTAs per tile, ring stages, MMA warps} of a projection on a device that holds fit[ks] clusters
@@ -210,7 +235,8 @@ cudaError_t launch_gate_up(photon_ctx *ctx, const ConvParams &p, cudaStream_t st
 // 8 rows, 4 heads at a time); -1 without a device
 int linear_slab_registers();
 int chunk_attn_registers();
-cudaError_t launch_rmsnorm(const bf16 *x, const bf16 *gamma, float eps, bf16 *out, int rows, int cols,
+// g.n > 0: the kernel does the work of launch_grow too (g.n at most rows)
+cudaError_t launch_rmsnorm(const bf16 *x, const bf16 *gamma, float eps, bf16 *out, int rows, int cols, const Grow &g,
                            cudaStream_t st, long long *launches);
 cudaError_t launch_rope_split(const bf16 *qkv, const int32_t *pos, int period, int n, int Hq, int Hkv, int dh,
                               float theta, bf16 *q, bf16 *k, bf16 *v, cudaStream_t st, long long *launches);
@@ -223,5 +249,13 @@ cudaError_t launch_read_probe(photon_ctx *ctx, const void *src, size_t bytes, in
                               cudaStream_t st, long long *launches);
 cudaError_t launch_wait_probe(photon_ctx *ctx, unsigned long long limit_ns, cudaStream_t st, long long *launches);
 
+__device__ __forceinline__ void grow_item(const Grow &g, int i) {
+    if (i >= g.n) return;
+    const int u = g.unit_ids ? __ldcg(g.unit_ids + i) : i;
+    if (u < 0 || u >= g.n_units) { atomicOr(g.status, PHOTON_DEV_BAD_INDEX); return; }
+    const int at = __ldcg(g.len + u);
+    if (at < 0 || at + g.n_rows > g.cap) { atomicOr(g.status, PHOTON_DEV_CAPACITY); return; }
+    g.len[u] = at + g.n_rows;
+}
 __device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }

@@ -24,11 +24,15 @@
 // columns; a tile is NT/2 gate columns and the NT/2 up columns of the same features, and silu(gate) * up goes
 // into U [B, F] (both rounded to bf16 first, as when they are stored and read back by the activation
 // kernel).  No bias, no residual.
+//
+// ROTARY: a fused q/k/v projection that leaves rotated, split and appended (see RopeOut).  A tile is one head; a group of columns is 8
+// features and their rotation partners.  The angles are computed where they are used, from the row's position.
 #include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
 #include "ptx.cuh"
+#include "rope.cuh"
 
 namespace {
 
@@ -54,6 +58,7 @@ constexpr int GROUP = 16;               // accumulator columns that change hands
 constexpr int QUAD_BYTES = 32 * GROUP * 4;          // a group's values of 32 rows
 constexpr int BAR_BYTES = 512;
 constexpr int RING_BYTES = 208 * 1024;
+constexpr int ANGLES_BYTES = 16 * 1024;             // ROTARY: cosines and sines of the first positions
 
 // First group of the part of a tile that CTA r of ks puts together.
 __host__ __device__ __forceinline__ int first_group(int groups, int r, int ks) { return groups * r / ks; }
@@ -63,24 +68,27 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     return *reinterpret_cast<uint32_t *>(&t);
 }
 
-// n groups of this warp's 32 rows from the accumulator (both: the sum of two); GATED: group g is 8 gate columns and the 8
-// up columns of the same features.
-template <int NT, bool GATED, int n>
+enum Epilogue { PLAIN, GATED_MLP, ROTARY };     // what a tile becomes
+
+// n groups of this warp's 32 rows from the accumulator (both: the sum of two).  HALVES: group g is 8 columns of the tile's first half
+// and the 8 of its second half that belong to them (gate and up columns of the same features; a feature and its rotation partner).
+template <int NT, bool HALVES, int n>
 __device__ __forceinline__ void load_groups(uint32_t acc, bool both, int g, uint32_t (&r)[n * GROUP]) {
-    if constexpr (GATED) {
+    auto load = [&](uint32_t from, uint32_t *to) {
 #pragma unroll
         for (int h = 0; h < n; ++h) {
-            ptx::tmem_ld_32x8(acc + (g + h) * (GROUP / 2), r + h * GROUP);
-            ptx::tmem_ld_32x8(acc + NT / 2 + (g + h) * (GROUP / 2), r + h * GROUP + GROUP / 2);
+            if constexpr (HALVES) {
+                ptx::tmem_ld_32x8(from + (g + h) * (GROUP / 2), to + h * GROUP);
+                ptx::tmem_ld_32x8(from + NT / 2 + (g + h) * (GROUP / 2), to + h * GROUP + GROUP / 2);
+            } else {
+                ptx::tmem_ld_32x16(from + (g + h) * GROUP, to + h * GROUP);
+            }
         }
-    } else {
-#pragma unroll
-        for (int h = 0; h < n; ++h) ptx::tmem_ld_32x16(acc + (g + h) * GROUP, r + h * GROUP);
-    }
+    };
+    load(acc, r);
     if constexpr (mma_warps(NT) == 2) {
         uint32_t r2[n * GROUP];
-#pragma unroll
-        for (int h = 0; h < n; ++h) ptx::tmem_ld_32x16(acc + NT + (g + h) * GROUP, r2 + h * GROUP);
+        load(acc + NT, r2);
         ptx::tmem_ld_wait();
         if (both)
 #pragma unroll
@@ -90,9 +98,10 @@ __device__ __forceinline__ void load_groups(uint32_t acc, bool both, int g, uint
     }
 }
 
-template <int NT, bool W_IN_MAJOR, bool GATED>
+template <int NT, bool W_IN_MAJOR, Epilogue EPI>
 __global__ void __launch_bounds__(SLAB_THREADS, min_ctas(NT))
 linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w) {
+    constexpr bool GATED = EPI == GATED_MLP, ROPE = EPI == ROTARY, HALVES = EPI != PLAIN;
     constexpr int W_BYTES = NT * BK * 2, GROUPS = NT / GROUP, KA = blocks_per_stage(NT), MW = mma_warps(NT), AT_ONCE = groups_at_once(NT);
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = ptx::smem_u32(smem_raw);
@@ -122,6 +131,10 @@ linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
         if (ks > 1) ptx::mbar_arrive_expect_tx(bar_rx, (ks - 1) * own * nq * QUAD_BYTES);
         ptx::prefetch_tmap(&tm_x); ptx::prefetch_tmap(&tm_w);
     }
+    double *inv = reinterpret_cast<double *>(smem_raw + RING_BYTES + BAR_BYTES);   // ROPE: a tile is one head, dh = NT
+    [[maybe_unused]] rope::Table angles{reinterpret_cast<float2 *>(inv + NT / 2), inv,
+                                        min(p.rope.period, ANGLES_BYTES / (rope::table_stride(NT) * 8)), NT / 2, rope::table_stride(NT)};
+    if (ROPE && threadIdx.x < NT / 2) inv[threadIdx.x] = rope::inverse_wavelength(threadIdx.x, NT, p.rope.log2_theta);
     if (warp == 1) ptx::tmem_alloc(ptx::smem_u32(const_cast<uint32_t *>(tmem_slot)), MW * NT);
     ptx::tc_fence_before();
     __syncthreads();
@@ -211,7 +224,9 @@ linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
             if (s >= p.stages) { s -= p.stages; phase ^= 1; }
         }
     }
+    if (ROPE && warp >= 2 && warp < 6) angles.fill(threadIdx.x - 64, 128);
     __syncwarp();
+    if (ROPE) __syncthreads();
 
     if (warp == 0) ptx::grid_dep_wait();                         // (the weights did not wait; what follows does)
 
@@ -228,7 +243,7 @@ linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
     // (4096 x 2048 -> 2048: 46.9 us, 42 since)
     uint4 res[AT_ONCE * GROUP / 8];
     auto fetch_residual = [&](int g) {
-        if constexpr (!GATED) {
+        if constexpr (EPI == PLAIN) {
             if (!p.residual || !live) return;
 #pragma unroll
             for (int v = 0; v < AT_ONCE * GROUP / 8; ++v)
@@ -237,6 +252,10 @@ linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
         }
     };
     fetch_residual(g_begin);
+    [[maybe_unused]] const rope::Row to = [&]() {
+        if (ROPE && live) return rope::Row(p.rope, b);
+        return rope::Row();
+    }();
     // one lane polls: 256 threads at the barrier hold up those that feed it (128 x 1024 -> 1024: 5.2 us, 5.0 with one)
     bool ok = lane != 0 || ptx::mbar_wait(bar_acc, 0);
     if (!ok) atomicOr(p.status, PHOTON_DEV_TIMEOUT);
@@ -249,7 +268,7 @@ linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
         if (quad < nq)
             for (int g = AT_ONCE * half; g < GROUPS; g += 2 * AT_ONCE) {   // the other CTAs' groups, in the order of their owners
                 uint32_t r[AT_ONCE * GROUP];
-                load_groups<NT, GATED, AT_ONCE>(acc, both, g, r);
+                load_groups<NT, HALVES, AT_ONCE>(acc, both, g, r);
 #pragma unroll
                 for (int h = 0; h < AT_ONCE; ++h) {
                     if (g + h >= g_lo && g + h < g_lo + own) continue;
@@ -288,7 +307,7 @@ linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
             uint32_t r[COLS], w[WORDS];
             [[maybe_unused]] const int col = n0 + g * GROUP;
             __syncwarp();                                  // rows past the batch took no part above, and left the round before early
-            load_groups<NT, GATED, n>(acc, both, g, r);
+            load_groups<NT, HALVES, n>(acc, both, g, r);
             for (int z = 0; z < ks - 1; ++z)
 #pragma unroll
                 for (int h = 0; h < n; ++h) {
@@ -304,6 +323,19 @@ linear_slab_kernel(const ConvParams p, const __grid_constant__ CUtensorMap tm_x,
                     }
                 }
             if (!live || !ok) return;
+            if constexpr (ROPE) {
+                constexpr int F = n * GROUP / 2;            // features, and as many partners
+                uint32_t lo[F], hi[F];
+#pragma unroll
+                for (int e = 0; e < F; ++e) {
+                    lo[e] = r[e / (GROUP / 2) * GROUP + e % (GROUP / 2)];
+                    hi[e] = r[e / (GROUP / 2) * GROUP + GROUP / 2 + e % (GROUP / 2)];
+                }
+                float cs[F], sn[F];
+                angles.get(to.at, g * (GROUP / 2), cs, sn);
+                rope::store<F>(p.rope, to, n0 / NT, g * (GROUP / 2), lo, hi, cs, sn);
+                return;
+            }
             bf16 *dst;
             if constexpr (GATED) {
 #pragma unroll
@@ -383,12 +415,13 @@ struct SlabPlan {
 // of 3, 18.7 as 96 CTAs; 300 x 2816 -> 1024 14.3 and 8.3; 1600 x 8192 -> 2048 80 as 104 clusters of 4, 47 unsplit.  Taken now, us with
 // weights ahead: 127 x 2048 -> 2048 7.2 as 32 tiles x 4 (8.3 unsplit), 127 x 5632 -> 2048 10.2 as 32 x 4 (17.7), 127 x 2048 ->
 // 3072 8.0 as 48 x 2 (8.3), 1204 x 2048 -> 2048 15.2 as 80 tiles of 256 columns (22.8 as 320 of 64).
-SlabPlan slab_plan(const int *fit, int B, int K, int N, int x_rows, bool gated) {
+// only: the one width that serves (0: all do)
+SlabPlan slab_plan(const int *fit, int B, int K, int N, int x_rows, int only) {
     const int m_tiles = (B + BM - 1) / BM, atoms = K / BK, nq = x_rows > 32 ? x_rows / 32 : 1;
     const float weights_us = (float)N * K * 2 / 5.75e6f, few_rows = 1.f - 0.08f * (float)(BM - x_rows) / BM;
     SlabPlan best{};
     for (int nt = 64; nt <= 256; nt *= 2) {
-        if (N % nt != 0 || (gated && nt != 128)) continue;
+        if (N % nt != 0 || (only && nt != only)) continue;
         const int groups = nt / GROUP;
         const float block_us = (nt == 64 ? 0.17f : nt == 128 ? 0.195f : 0.255f) * few_rows;
         for (int ks = 1; ks <= MAX_CLUSTER && ks <= groups && ks * 2 <= std::max(2, atoms); ++ks) {
@@ -409,49 +442,47 @@ SlabPlan slab_plan(const int *fit, int B, int K, int N, int x_rows, bool gated) 
 
 int rows_fetched(int B) { return B > 64 ? 128 : B > 32 ? 64 : B > 16 ? 32 : 16; }
 
-template <int NT, bool IN_MAJOR, bool GATED>
+int only_width(const ConvParams &p, bool gated) { return gated ? 128 : p.rope.q ? p.rope.dh : 0; }
+
+template <int NT, bool IN_MAJOR, Epilogue EPI>
 cudaError_t run_as(photon_ctx *ctx, ConvParams p, const SlabPlan &s, cudaStream_t st, long long *launches) {
     const CUtensorMap *t;
     CUtensorMap mx, mw;
     if (!(t = ctx->tmaps.get(p.x, (uint64_t)p.B, (uint64_t)p.D, p.x_rows))) return cudaErrorInvalidValue;
     mx = *t;
     // [K, N] in boxes of 64 k x 64 n, or [N, K] in boxes of NT n x 64 k (gate rows and up rows are fetched apart)
-    t = IN_MAJOR ? ctx->tmaps.get(p.w, (uint64_t)p.D, (uint64_t)p.N, BK) : ctx->tmaps.get(p.w, (uint64_t)p.N, (uint64_t)p.D, GATED ? NT / 2 : NT);
+    t = IN_MAJOR ? ctx->tmaps.get(p.w, (uint64_t)p.D, (uint64_t)p.N, BK) : ctx->tmaps.get(p.w, (uint64_t)p.N, (uint64_t)p.D, EPI == GATED_MLP ? NT / 2 : NT);
     if (!t) return cudaErrorInvalidValue;
     mw = *t;
     p.ksplit = s.ks; p.stages = s.stages;
     p.once = p.w_ahead && (p.D / BK + s.ks - 1) / s.ks <= s.stages * blocks_per_stage(NT);
-    constexpr size_t smem = (size_t)RING_BYTES + BAR_BYTES;
+    constexpr size_t smem = (size_t)RING_BYTES + BAR_BYTES + (EPI == ROTARY ? NT / 2 * sizeof(double) + ANGLES_BYTES : 0);
     static size_t smem_set[kMaxDevices] = {};
-    if (const cudaError_t e = ensure_dynamic_smem(linear_slab_kernel<NT, IN_MAJOR, GATED>, smem, ctx->device, smem_set)) return e;
+    if (const cudaError_t e = ensure_dynamic_smem(linear_slab_kernel<NT, IN_MAJOR, EPI>, smem, ctx->device, smem_set)) return e;
     const dim3 grid(p.ksplit * (p.N / NT), (p.B + BM - 1) / BM);
-    const cudaError_t e = launch_dependent(linear_slab_kernel<NT, IN_MAJOR, GATED>, grid, dim3(SLAB_THREADS), smem, st,
+    const cudaError_t e = launch_dependent(linear_slab_kernel<NT, IN_MAJOR, EPI>, grid, dim3(SLAB_THREADS), smem, st,
                                            p.ksplit > 1 ? p.ksplit : 0, p, mx, mw);
     ++*launches;
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <bool GATED>
+template <Epilogue EPI>
 cudaError_t run(photon_ctx *ctx, ConvParams p, cudaStream_t st, long long *launches) {
     if (p.B == 0) return cudaSuccess;
     p.x_rows = rows_fetched(p.B);
-    const SlabPlan s = slab_plan(ctx->clusters, p.B, p.D, p.N, p.x_rows, GATED);
-    if constexpr (GATED) {
-        if (s.nt != 128) return cudaErrorInvalidValue;
-        return p.w_out_major ? run_as<128, false, true>(ctx, p, s, st, launches) : run_as<128, true, true>(ctx, p, s, st, launches);
-    } else {
-        if (p.w_out_major)
-            return s.nt == 256 ? run_as<256, false, false>(ctx, p, s, st, launches)
-                               : s.nt == 128 ? run_as<128, false, false>(ctx, p, s, st, launches) : run_as<64, false, false>(ctx, p, s, st, launches);
-        return s.nt == 256 ? run_as<256, true, false>(ctx, p, s, st, launches)
-                           : s.nt == 128 ? run_as<128, true, false>(ctx, p, s, st, launches) : run_as<64, true, false>(ctx, p, s, st, launches);
-    }
+    const SlabPlan s = slab_plan(ctx->clusters, p.B, p.D, p.N, p.x_rows, only_width(p, EPI == GATED_MLP));
+    if constexpr (EPI != GATED_MLP)
+        if (s.nt == 64) return p.w_out_major ? run_as<64, false, EPI>(ctx, p, s, st, launches) : run_as<64, true, EPI>(ctx, p, s, st, launches);
+    if (s.nt == 128) return p.w_out_major ? run_as<128, false, EPI>(ctx, p, s, st, launches) : run_as<128, true, EPI>(ctx, p, s, st, launches);
+    if constexpr (EPI == PLAIN)
+        if (s.nt == 256) return p.w_out_major ? run_as<256, false, EPI>(ctx, p, s, st, launches) : run_as<256, true, EPI>(ctx, p, s, st, launches);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
 cudaError_t launch_linear(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches) {
-    return run<false>(ctx, p, st, launches);
+    return run<PLAIN>(ctx, p, st, launches);
 }
 
 // Whether the fused gate/up form serves this shape: whole slabs of 64 features, and enough of them to occupy half of the
@@ -461,8 +492,12 @@ bool gate_up_fits_small_tiles(const photon_ctx *ctx, const ConvParams &p) {
     return p.N % 128 == 0 && p.D % BK == 0 && tiles * 2 >= ctx->sm_count;
 }
 
+cudaError_t launch_qkv_rope(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches) {
+    return run<ROTARY>(ctx, p, st, launches);
+}
+
 cudaError_t launch_gate_up(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches) {
-    return run<true>(ctx, p, st, launches);
+    return run<GATED_MLP>(ctx, p, st, launches);
 }
 
 // How many clusters of 1 to MAX_CLUSTER CTAs of this kernel the device holds at a time.  Asked once per device: the eight
@@ -475,7 +510,7 @@ cudaError_t linear_cluster_counts(int device, int (&fit)[MAX_CLUSTER + 1]) {
         return cudaSuccess;
     }
     constexpr size_t smem = (size_t)RING_BYTES + BAR_BYTES;
-    const auto kernel = linear_slab_kernel<64, true, false>;         // (the other forms take as much of everything that counts here)
+    const auto kernel = linear_slab_kernel<64, true, PLAIN>;         // (the other forms take as much of everything that counts here)
     if (const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return e;
     fit[0] = 0;
     for (int ks = 1; ks <= MAX_CLUSTER; ++ks) {
@@ -499,18 +534,18 @@ cudaError_t linear_cluster_counts(int device, int (&fit)[MAX_CLUSTER + 1]) {
 // The estimate above was fitted to small batches; with the whole chip at work the same cuts take about a quarter longer,
 // every wave ends in an epilogue of its own, and the residual and the output move while nothing else does (5 TB/s).
 float linear_slab_us(const int *fit, const ConvParams &p, bool gated) {
-    const SlabPlan s = slab_plan(fit, p.B, p.D, p.N, rows_fetched(p.B), gated);
+    const SlabPlan s = slab_plan(fit, p.B, p.D, p.N, rows_fetched(p.B), only_width(p, gated));
     if (s.nt == 0) return -1.f;
     const long long tiles = (long long)(p.N / s.nt) * ((p.B + BM - 1) / BM), waves = (tiles + fit[s.ks] - 1) / fit[s.ks];
     return 1.25f * s.us + waves * (s.nt / 256.f) + (float)p.B * p.N * (p.residual ? 4 : 2) / 5e6f;
 }
 
 void linear_cut(const int *fit, int B, int K, int N, bool gated, int32_t *cut) {
-    const SlabPlan s = slab_plan(fit, B, K, N, rows_fetched(B), gated);
+    const SlabPlan s = slab_plan(fit, B, K, N, rows_fetched(B), gated ? 128 : 0);
     cut[0] = s.nt; cut[1] = s.ks; cut[2] = s.stages; cut[3] = mma_warps(s.nt);
 }
 
 int linear_slab_registers() {
     cudaFuncAttributes a{};
-    return cudaFuncGetAttributes(&a, linear_slab_kernel<64, false, false>) == cudaSuccess ? (a.numRegs + 7) / 8 * 8 * SLAB_THREADS : -1;
+    return cudaFuncGetAttributes(&a, linear_slab_kernel<64, false, PLAIN>) == cudaSuccess ? (a.numRegs + 7) / 8 * 8 * SLAB_THREADS : -1;
 }

@@ -18,6 +18,7 @@
 
 #include "common.cuh"
 #include "ptx.cuh"
+#include "rope.cuh"
 
 namespace {
 
@@ -62,7 +63,7 @@ rope_split_kernel(const bf16 *qkv, const int32_t *pos, int period, int n, int Hq
     __shared__ __align__(16) float cs[2][128], sn[2][128];
     const int half = dh / 2, vec_half = half / 8;        // 16-byte pieces per half head
     const int j0 = (threadIdx.x % vec_half) * 8;         // 256 is a multiple of vec_half: the same features for every piece
-    const double inv = exp2(-2.0 * (double)threadIdx.x / dh * log2_theta);
+    const double inv = rope::inverse_wavelength(threadIdx.x, dh, log2_theta);
     const int rotated = (Hq + Hkv) * vec_half, copied = Hkv * dh / 8;
     const int width = (Hq + 2 * Hkv) * dh, step = gridDim.x;
     ptx::grid_dep_wait();                   // qkv is the output of the kernel before this one
@@ -72,12 +73,7 @@ rope_split_kernel(const bf16 *qkv, const int32_t *pos, int period, int n, int Hq
     // never releases its dependents early either) the attention starts with a clean L1.
     if (!APPEND) ptx::grid_dep_launch();
     auto where = [&](int i) { return i < n ? (pos ? pos[i] : i % period) : 0; };   // no position array: row i % period of its group
-    auto table = [&](int at, int buf) {
-        // the angle and its reduction to [-pi, pi] in double precision, sine and cosine of the remainder in single
-        const double a = (double)at * inv;
-        const double turns = rint(a * 0.15915494309189535);
-        __sincosf((float)fma(turns, -6.283185307179586, a), &sn[buf][threadIdx.x], &cs[buf][threadIdx.x]);
-    };
+    auto table = [&](int at, int buf) { rope::angle(at, inv, &cs[buf][threadIdx.x], &sn[buf][threadIdx.x]); };
     const bool tabler = (int)threadIdx.x < half;
     int at = where(blockIdx.x), at_next = where(blockIdx.x + step);
     if (tabler) table(at, 0);
@@ -166,7 +162,22 @@ swiglu_kernel(const bf16 *gu, bf16 *out, int n, int F) {
     }
 }
 
+// The lengths that go with keys and values that a projection's epilogue has written.
+__global__ void __launch_bounds__(EW_THREADS)
+grow_kernel(const Grow g) {
+    ptx::grid_dep_wait();                   // the kernel before this one reads the lengths
+    ptx::grid_dep_launch();
+    grow_item(g, blockIdx.x * EW_THREADS + threadIdx.x);
+}
+
 }  // namespace
+
+cudaError_t launch_grow(const Grow &g, cudaStream_t st, long long *launches) {
+    if (g.n == 0) return cudaSuccess;
+    const cudaError_t e = launch_dependent(grow_kernel, dim3((g.n + EW_THREADS - 1) / EW_THREADS), dim3(EW_THREADS), 0, st, 0, g);
+    ++*launches;
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
 
 cudaError_t launch_rope_split(const bf16 *qkv, const int32_t *pos, int period, int n, int Hq, int Hkv, int dh,
                               float theta, bf16 *q, bf16 *k, bf16 *v, cudaStream_t st, long long *launches) {

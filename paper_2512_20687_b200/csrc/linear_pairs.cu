@@ -24,10 +24,13 @@
 // GATED: the gate/up projection of the MLP with its activation folded in.  The weight is [gate | up] (N = 2F columns); a
 // tile takes as many gate columns as up columns of the same features: the first CTA brings the gate half, the second
 // the up half, and the epilogue writes silu(g) * u: out [B, F], and the [B, 2F] intermediate never exists.
+//
+// ROTARY: a fused q/k/v projection that leaves rotated, split and appended (see RopeOut); tiles are whole heads.
 #include <algorithm>
 
 #include "common.cuh"
 #include "ptx.cuh"
+#include "rope.cuh"
 
 namespace {
 
@@ -37,6 +40,12 @@ constexpr int RING = 196 * 1024, MAX_STAGES = 8;     // 6, 7 or 8 stages of 256,
 constexpr int EPI_PARTS = 2, EPI_WARPS = 4 * EPI_PARTS;
 constexpr int LL_THREADS = 128 + EPI_WARPS * 32;    // warp 0: weights, warp 1: MMA (owns TMEM), warp 2: x, warps 4..: epilogue
 constexpr int LL_SMEM = RING + 1024 + 256;
+// ROTARY: a ring of 192 KB, inverse wavelengths (up to 64 doubles), and cosines and sines of up to 64 positions
+constexpr int RING_ROTARY = 192 * 1024, INV_AT = RING_ROTARY + 256, TABLE_BYTES = 64 * (64 + 1) * 8;
+constexpr int LL_SMEM_ROTARY = RING_ROTARY + 1024 + 256 + 64 * 8 + TABLE_BYTES;
+__host__ __device__ constexpr int ring_bytes(bool rotary) { return rotary ? RING_ROTARY : RING; }
+
+enum Epilogue { PLAIN, GATED_MLP, ROTARY };         // what a tile becomes
 
 // How the output is cut: tiles of 256 rows x nt columns; the pieces of a call are `whole` tiles and then the two halves of
 // each further tile.
@@ -65,17 +74,19 @@ __device__ __forceinline__ Piece piece_at(const ConvParams &p, const PairPlan &c
     return x;
 }
 
-template <bool W_IN_MAJOR, bool GATED>
+template <bool W_IN_MAJOR, Epilogue EPI>
 __global__ void __launch_bounds__(LL_THREADS, 1)
 linear_pair_kernel(const ConvParams p, const PairPlan c, const __grid_constant__ CUtensorMap tm_x,
                    const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_w_half) {
+    constexpr bool GATED = EPI == GATED_MLP;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;     // (the same in both CTAs)
     uint8_t *gen = smem_raw + (base - ptx::smem_u32(smem_raw));
-    const uint32_t full = base + RING, empty = full + 8 * MAX_STAGES;         // full: the first CTA's are used, for both
+    constexpr int RING_END = ring_bytes(EPI == ROTARY);
+    const uint32_t full = base + RING_END, empty = full + 8 * MAX_STAGES;         // full: the first CTA's are used, for both
     const uint32_t acc_full = empty + 8 * MAX_STAGES, acc_empty = acc_full + 16;   // [2] each; acc_empty: the first CTA's
-    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(gen + RING + 16 * MAX_STAGES + 32);
-    volatile int *dead = reinterpret_cast<volatile int *>(gen + RING + 16 * MAX_STAGES + 40);
+    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(gen + RING_END + 16 * MAX_STAGES + 32);
+    volatile int *dead = reinterpret_cast<volatile int *>(gen + RING_END + 16 * MAX_STAGES + 40);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = blockIdx.x & 1, pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
@@ -96,6 +107,8 @@ linear_pair_kernel(const ConvParams p, const PairPlan c, const __grid_constant__
         ptx::prefetch_tmap(&tm_x); ptx::prefetch_tmap(&tm_w);
         if (c.pieces > c.whole) ptx::prefetch_tmap(&tm_w_half);
     }
+    double *inv = reinterpret_cast<double *>(gen + INV_AT);
+    if (EPI == ROTARY && threadIdx.x < p.rope.dh / 2) inv[threadIdx.x] = rope::inverse_wavelength(threadIdx.x, p.rope.dh, p.rope.log2_theta);
     if (warp == 1) ptx::tmem_alloc_pair(ptx::smem_u32(const_cast<uint32_t *>(tmem_slot)), 2 * NT_MAX);
     ptx::tc_fence_before();
     __syncthreads();
@@ -192,6 +205,11 @@ linear_pair_kernel(const ConvParams p, const PairPlan c, const __grid_constant__
             *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
             *reinterpret_cast<uint4 *>(dst + 8) = make_uint4(w[4], w[5], w[6], w[7]);
         };
+        [[maybe_unused]] rope::Table angles{reinterpret_cast<float2 *>(inv + 64), inv, rope::positions(p.rope), p.rope.dh / 2, rope::table_stride(p.rope.dh)};
+        if constexpr (EPI == ROTARY) {
+            angles.fill(threadIdx.x - 128, 32 * EPI_WARPS);
+            ptx::named_bar_sync(1, 32 * EPI_WARPS);
+        }
         int n = 0;
         for (int i = pair; i < c.pieces && !*dead; i += pairs, ++n) {
             const int buf = n & 1;
@@ -199,8 +217,8 @@ linear_pair_kernel(const ConvParams p, const PairPlan c, const __grid_constant__
             const int b = x.m0 + rank * BM + quad * 32 + lane;
             const bool live = b < p.B;
             constexpr int ROUNDS = NT_MAX / (32 * EPI_PARTS);                   // groups of 32 columns per warp, at most
-            [[maybe_unused]] uint4 res[GATED ? 1 : ROUNDS][4];
-            if constexpr (!GATED) {
+            [[maybe_unused]] uint4 res[EPI == PLAIN ? ROUNDS : 1][4];
+            if constexpr (EPI == PLAIN) {
                 if (p.residual && live) {
                     const bf16 *row = p.residual + (size_t)b * p.N + x.n0;
 #pragma unroll
@@ -212,6 +230,8 @@ linear_pair_kernel(const ConvParams p, const PairPlan c, const __grid_constant__
                     }
                 }
             }
+            [[maybe_unused]] rope::Row to;
+            if (EPI == ROTARY && live) to = rope::Row(p.rope, b);
             // one lane polls, and not all the time: polling takes issue slots and barrier accesses from the warps that feed the MMAs
             bool ok = lane != 0 || ptx::mbar_wait_idle(acc_full + 8 * buf, (n >> 1) & 1);
             ok = __shfl_sync(0xffffffffu, (int)ok, 0);
@@ -238,6 +258,24 @@ linear_pair_kernel(const ConvParams p, const PairPlan c, const __grid_constant__
                         w[e] = *reinterpret_cast<const uint32_t *>(&o);
                     }
                     store(p.U + (size_t)b * n_out + x.n0 + f, w);
+                }
+            } else if constexpr (EPI == ROTARY) {
+                // 16 feature pairs at a time, for all heads of the piece: their angles are the same
+                const int dh = p.rope.dh;
+#pragma unroll 1
+                for (int j = 16 * part; j < dh / 2; j += 16 * EPI_PARTS) {
+                    float cs[16], sn[16];
+                    angles.get(to.at, j, cs, sn);
+                    int h = x.n0 / dh;
+#pragma unroll 1
+                    for (int c0 = 0; c0 < x.width; c0 += dh, ++h) {
+                        uint32_t lo[16], hi[16];
+                        __syncwarp();                                           // (likewise)
+                        ptx::tmem_ld_32x16(lanes + buf * NT_MAX + c0 + j, lo);
+                        ptx::tmem_ld_32x16(lanes + buf * NT_MAX + c0 + dh / 2 + j, hi);
+                        ptx::tmem_ld_wait();
+                        if (live && x.n0 + c0 < n_out) rope::store<16>(p.rope, to, h, j, lo, hi, cs, sn);
+                    }
                 }
             } else {
 #pragma unroll
@@ -293,14 +331,16 @@ linear_pair_kernel(const ConvParams p, const PairPlan c, const __grid_constant__
 // 2048 -> 11264: 35.6 with the last round of 28 tiles in halves, 36.9 without.
 float block_us(int width) { return width >= 256 ? 0.30f : width >= 192 ? 0.235f : width >= 128 ? 0.215f : 0.21f; }
 
-PairPlan pair_plan(int pairs, int B, int K, int N, bool in_major) {
+// grain: what tiles and halves have to be multiples of (0: nothing)
+PairPlan pair_plan(int pairs, int B, int K, int N, bool in_major, int grain) {
     PairPlan best{};
     for (int nt = NT_MAX; nt >= 128; nt -= 64) {
+        if (grain && nt % grain != 0) continue;
         const int w_cols = in_major ? (nt / 2 + 63) / 64 * 64 : nt / 2;     // N-major weights come in boxes of 64 columns
         const int stage_bytes = A_BYTES + w_cols * BK * 2, atoms = K / BK;
-        PairPlan c{nt, (B + 2 * BM - 1) / (2 * BM), (N + nt - 1) / nt, 0, 0, std::min(MAX_STAGES, RING / stage_bytes), stage_bytes, 0, 0.f};
+        PairPlan c{nt, (B + 2 * BM - 1) / (2 * BM), (N + nt - 1) / nt, 0, 0, std::min(MAX_STAGES, ring_bytes(grain > 0) / stage_bytes), stage_bytes, 0, 0.f};
         const int tiles = c.m_tiles * c.n_tiles, rounds = tiles / pairs, rest = tiles % pairs;
-        const bool halves = rest > 0 && 2 * rest <= pairs;
+        const bool halves = rest > 0 && 2 * rest <= pairs && !(grain && nt / 2 % grain != 0);
         const int last = rest == 0 || (halves && rounds > 0) ? nt : halves ? nt / 2 : nt;
         c.us = rounds * (atoms * block_us(nt) + 1.2f) + (rest ? atoms * block_us(halves ? nt / 2 : nt) : 0.f) +
                (last >= 256 ? 5.6f : last >= 192 ? 4.9f : 4.1f);
@@ -312,13 +352,16 @@ PairPlan pair_plan(int pairs, int B, int K, int N, bool in_major) {
     return best;
 }
 
-template <bool IN_MAJOR, bool GATED>
+int grain_of(const ConvParams &p) { return p.rope.q ? p.rope.dh : 0; }
+
+template <bool IN_MAJOR, Epilogue EPI>
 cudaError_t run_large(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches) {
     static size_t smem_set[kMaxDevices] = {};
-    if (const cudaError_t e = ensure_dynamic_smem(linear_pair_kernel<IN_MAJOR, GATED>, LL_SMEM, ctx->device, smem_set)) return e;
+    constexpr size_t smem = EPI == ROTARY ? LL_SMEM_ROTARY : LL_SMEM;
+    if (const cudaError_t e = ensure_dynamic_smem(linear_pair_kernel<IN_MAJOR, EPI>, smem, ctx->device, smem_set)) return e;
     if (p.B == 0) return cudaSuccess;
     const int pairs = ctx->clusters[2];
-    const PairPlan c = pair_plan(pairs, p.B, p.D, p.N, IN_MAJOR);
+    const PairPlan c = pair_plan(pairs, p.B, p.D, p.N, IN_MAJOR, grain_of(p));
     const CUtensorMap *t;
     CUtensorMap mx, mw, mw_half;
     if (!(t = ctx->tmaps.get(p.x, (uint64_t)p.B, (uint64_t)p.D, BM))) return cudaErrorInvalidValue;
@@ -331,8 +374,8 @@ cudaError_t run_large(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, lon
         if (!(t = ctx->tmaps.get(p.w, (uint64_t)p.N, (uint64_t)p.D, c.nt / 4))) return cudaErrorInvalidValue;
         mw_half = *t;
     }
-    const cudaError_t e = launch_dependent(linear_pair_kernel<IN_MAJOR, GATED>, dim3(2 * std::min(c.pieces, pairs)),
-                                           dim3(LL_THREADS), LL_SMEM, st, 2, p, c, mx, mw, mw_half);
+    const cudaError_t e = launch_dependent(linear_pair_kernel<IN_MAJOR, EPI>, dim3(2 * std::min(c.pieces, pairs)),
+                                           dim3(LL_THREADS), smem, st, 2, p, c, mx, mw, mw_half);
     ++*launches;
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -345,21 +388,25 @@ cudaError_t run_large(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, lon
 bool linear_wants_pairs(const int *fit, const ConvParams &p, bool gated) {
     if (fit[2] < 1 || p.B <= BM) return false;
     const float slab = linear_slab_us(fit, p, gated);
-    return slab < 0.f || 1.04f * pair_plan(fit[2], p.B, p.D, p.N, !p.w_out_major).us < slab;
+    return slab < 0.f || 1.04f * pair_plan(fit[2], p.B, p.D, p.N, !p.w_out_major, grain_of(p)).us < slab;
 }
 
 void linear_pair_cut(const int *fit, const ConvParams &p, bool gated, int32_t *cut) {
-    const PairPlan c = pair_plan(std::max(1, fit[2]), p.B, p.D, p.N, !p.w_out_major);
+    const PairPlan c = pair_plan(std::max(1, fit[2]), p.B, p.D, p.N, !p.w_out_major, grain_of(p));
     const int32_t v[] = {linear_wants_pairs(fit, p, gated), c.nt, c.m_tiles, c.n_tiles, c.whole, c.pieces, c.stages, c.stage_bytes};
     std::copy(v, v + 8, cut);
 }
 
 cudaError_t launch_linear_pairs(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches) {
-    return p.w_out_major ? run_large<false, false>(ctx, p, st, launches) : run_large<true, false>(ctx, p, st, launches);
+    return p.w_out_major ? run_large<false, PLAIN>(ctx, p, st, launches) : run_large<true, PLAIN>(ctx, p, st, launches);
+}
+
+cudaError_t launch_qkv_rope_pairs(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches) {
+    return p.w_out_major ? run_large<false, ROTARY>(ctx, p, st, launches) : run_large<true, ROTARY>(ctx, p, st, launches);
 }
 
 // out [B, F] = silu(x Wg) * (x Wu) for w = [Wg | Wu] with N = 2F columns; for the shapes
 // linear_wants_pairs accepts.  No bias, no residual.
 cudaError_t launch_gate_up_pairs(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, long long *launches) {
-    return p.w_out_major ? run_large<false, true>(ctx, p, st, launches) : run_large<true, true>(ctx, p, st, launches);
+    return p.w_out_major ? run_large<false, GATED_MLP>(ctx, p, st, launches) : run_large<true, GATED_MLP>(ctx, p, st, launches);
 }

@@ -1,6 +1,7 @@
 // C boundary: context management, argument validation, launch sequencing.
 #include <chrono>
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <new>
 
@@ -237,9 +238,10 @@ photon_status photon_chunk_attn(photon_ctx *ctx, const photon_kv *chunks, const 
                             static_cast<cudaStream_t>(stream));
 }
 
-photon_status photon_chunk_causal_attn(photon_ctx *ctx, const photon_kv *chunks, const photon_bf16 *q,
-                                       const int32_t *slot, photon_bf16 *out, int32_t Nc, int32_t row0,
-                                       int32_t rows, float scale, photon_stream stream) {
+namespace {
+// grown: see CausalParams
+photon_status chunk_causal_attn(photon_ctx *ctx, const photon_kv *chunks, const photon_bf16 *q, const int32_t *slot, photon_bf16 *out,
+                                int32_t Nc, int32_t row0, int32_t rows, float scale, int grown, photon_stream stream) {
     if (!ctx || !chunks) return PHOTON_ERR_INVALID_ARG;
     if (!kv_ok(ctx, chunks, false) || chunks->page_table) return PHOTON_ERR_INVALID_ARG;
     if (chunks->cap > ctx->cfg.P + ctx->cfg.C || chunks->cap > 64) return PHOTON_ERR_INVALID_ARG;
@@ -249,6 +251,7 @@ photon_status photon_chunk_causal_attn(photon_ctx *ctx, const photon_kv *chunks,
     if (!aligned16(q) || !aligned16(out) || !(scale == scale)) return PHOTON_ERR_INVALID_ARG;
     const photon_config &c = ctx->cfg;
     CausalParams p{};
+    p.grown = grown;
     p.q = reinterpret_cast<const bf16 *>(q);
     p.out = reinterpret_cast<bf16 *>(out);
     p.k = reinterpret_cast<const bf16 *>(chunks->k);
@@ -262,6 +265,13 @@ photon_status photon_chunk_causal_attn(photon_ctx *ctx, const photon_kv *chunks,
     p.status = ctx->status;
     const cudaError_t e = launch_chunk_causal_attention(ctx, p, static_cast<cudaStream_t>(stream), &ctx->launches);
     return e == cudaSuccess ? PHOTON_OK : PHOTON_ERR_CUDA;
+}
+}  // namespace
+
+photon_status photon_chunk_causal_attn(photon_ctx *ctx, const photon_kv *chunks, const photon_bf16 *q,
+                                       const int32_t *slot, photon_bf16 *out, int32_t Nc, int32_t row0,
+                                       int32_t rows, float scale, photon_stream stream) {
+    return chunk_causal_attn(ctx, chunks, q, slot, out, Nc, row0, rows, scale, 0, stream);
 }
 
 namespace {
@@ -327,7 +337,7 @@ photon_status photon_rmsnorm(photon_ctx *ctx, const photon_bf16 *x, const photon
     if (rows > 0 && (!x || !out)) return PHOTON_ERR_INVALID_ARG;
     if (!aligned16(x) || !aligned16(gamma) || !aligned16(out) || !(eps >= 0.f)) return PHOTON_ERR_INVALID_ARG;
     const cudaError_t e = launch_rmsnorm(reinterpret_cast<const bf16 *>(x), reinterpret_cast<const bf16 *>(gamma), eps,
-                                         reinterpret_cast<bf16 *>(out), rows, cols,
+                                         reinterpret_cast<bf16 *>(out), rows, cols, Grow{},
                                          static_cast<cudaStream_t>(stream), &ctx->launches);
     return e == cudaSuccess ? PHOTON_OK : PHOTON_ERR_CUDA;
 }
@@ -390,6 +400,37 @@ photon_status gate_up(photon_ctx *ctx, const photon_layer *L, const photon_layer
     return s;
 }
 
+// The q/k/v projection of `rows` normalised rows with everything up to the attention in its epilogue: rotated queries in sc->q, keys
+// and values in the rows of the (contiguous) cache.
+ConvParams qkv_rope_params(photon_ctx *ctx, const photon_layer *L, const photon_layer_scratch *sc, int rows, photon_kv *cache,
+                           const int32_t *unit_ids, int period) {
+    const photon_config &c = ctx->cfg;
+    ConvParams p{};
+    p.x = reinterpret_cast<const bf16 *>(sc->n);
+    p.w = reinterpret_cast<const bf16 *>(L->wqkv);
+    p.U = reinterpret_cast<bf16 *>(sc->qkv);
+    p.B = rows; p.D = c.D; p.N = (c.Hq + 2 * c.Hkv) * c.dh;
+    p.w_out_major = (L->w_layout == PHOTON_W_OUT_MAJOR);
+    p.w_ahead = true;
+    p.status = ctx->status;
+    p.rope.q = reinterpret_cast<bf16 *>(sc->q);
+    p.rope.k_cache = reinterpret_cast<bf16 *>(cache->k);
+    p.rope.v_cache = reinterpret_cast<bf16 *>(cache->v);
+    p.rope.len = cache->len; p.rope.unit_ids = unit_ids;
+    p.rope.n_units = cache->n_units; p.rope.cap = cache->cap; p.rope.period = period;
+    p.rope.Hq = c.Hq; p.rope.Hkv = c.Hkv; p.rope.dh = c.dh;
+    p.rope.log2_theta = std::log2((double)L->theta);
+    return p;
+}
+photon_status qkv_rope(photon_ctx *ctx, const ConvParams &p, bool pairs, photon_stream stream) {
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const cudaError_t e = pairs ? launch_qkv_rope_pairs(ctx, p, st, &ctx->launches) : launch_qkv_rope(ctx, p, st, &ctx->launches);
+    return e == cudaSuccess ? PHOTON_OK : PHOTON_ERR_CUDA;
+}
+Grow grow_of(photon_ctx *ctx, const photon_kv *cache, const int32_t *unit_ids, int n, int n_rows) {
+    return Grow{cache->len, unit_ids, cache->n_units, cache->cap, n, n_rows, ctx->status};
+}
+
 // STEP of one layer for the newest position of every unit of `cache`; local: the cache is a set of chunk
 // buffers read by the chunk attention, else a coarse stream read by the coarse attention.
 photon_status layer_step(photon_ctx *ctx, const photon_layer *L, const photon_layer_scratch *sc,
@@ -410,8 +451,19 @@ photon_status layer_step(photon_ctx *ctx, const photon_layer *L, const photon_la
     if (!local && (size_t)B * c.Hkv > ctx->n_tickets) return PHOTON_ERR_WORKSPACE;
     if (local && (cache->cap > c.P + c.C || cache->page_table)) return PHOTON_ERR_INVALID_ARG;
     photon_status s = photon_rmsnorm(ctx, x, L->g1, L->eps, sc->n, B, D, stream);
-    if (s == PHOTON_OK) s = linear(ctx, sc->n, L->wqkv, L->w_layout, nullptr, nullptr, sc->qkv, B, D, QKV, true, stream);
-    if (s == PHOTON_OK) {
+    // Many chunks: the projection's epilogue rotates, splits and appends, and the projection itself (sc->qkv, 100 MB written and read
+    // back with 16384 chunks of width 1024) is not written: projection and split 127 us, 75 so.  Few: a cut into whole heads costs
+    // the small kernel about as much as the split kernel.
+    const ConvParams qkv = qkv_rope_params(ctx, L, sc, B, cache, nullptr, 0);
+    const bool fused = local && linear_wants_pairs(ctx->clusters, qkv, false);
+    if (fused) {
+        if (s == PHOTON_OK) s = qkv_rope(ctx, qkv, true, stream);
+        if (s == PHOTON_OK && launch_grow(grow_of(ctx, cache, nullptr, B, 1), static_cast<cudaStream_t>(stream), &ctx->launches) != cudaSuccess)
+            s = PHOTON_ERR_CUDA;
+    } else if (s == PHOTON_OK) {
+        s = linear(ctx, sc->n, L->wqkv, L->w_layout, nullptr, nullptr, sc->qkv, B, D, QKV, true, stream);
+    }
+    if (s == PHOTON_OK && !fused) {
         // split, rotation by the unit's length and the append in one kernel: k and v go straight into the cache rows
         const cudaError_t e = launch_rope_split_append(
             reinterpret_cast<const bf16 *>(sc->qkv), B, c.Hq, c.Hkv, c.dh, L->theta, reinterpret_cast<bf16 *>(sc->q),
@@ -454,19 +506,22 @@ photon_status photon_decoder_prefill(photon_ctx *ctx, const photon_layer *L, con
     for (const void *q : ptrs)
         if (!q || !aligned16(q)) return PHOTON_ERR_INVALID_ARG;
     if (n == 0) return PHOTON_OK;
-    const int P = c.P, T = n * P, D = c.D, QKV = (c.Hq + 2 * c.Hkv) * c.dh;      // T rows: the P prefix vectors of n chunks
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const int P = c.P, T = n * P, D = c.D;                                       // T rows: the P prefix vectors of n chunks
     photon_status s = photon_rmsnorm(ctx, U, L->g1, L->eps, sc->n, T, D, stream);
-    if (s == PHOTON_OK) s = linear(ctx, sc->n, L->wqkv, L->w_layout, nullptr, nullptr, sc->qkv, T, D, QKV, true, stream);
-    if (s == PHOTON_OK &&
-        launch_rope_split(reinterpret_cast<const bf16 *>(sc->qkv), nullptr, P, T, c.Hq, c.Hkv, c.dh, L->theta,
-                          reinterpret_cast<bf16 *>(sc->q), reinterpret_cast<bf16 *>(sc->k_new),
-                          reinterpret_cast<bf16 *>(sc->v_new), st, &ctx->launches) != cudaSuccess)
-        s = PHOTON_ERR_CUDA;
-    if (s == PHOTON_OK) s = photon_kv_append(ctx, chunks, sc->k_new, sc->v_new, unit_ids, n, P, stream);
-    if (s == PHOTON_OK) s = photon_chunk_causal_attn(ctx, chunks, sc->q, unit_ids, sc->att, n, 0, P, scale, stream);
+    // one projection that rotates, splits and appends, instead of three kernels (a trip between kernels each; 64 chunks of 4 rows, 2048
+    // wide, 64.4 -> 62.2 us, 200 of 8 rows, 1024 wide, 88.6 -> 78.2); the intermediates are written all the same
+    ConvParams qkv = qkv_rope_params(ctx, L, sc, T, chunks, unit_ids, P);
+    qkv.rope.qkv = reinterpret_cast<bf16 *>(sc->qkv);
+    qkv.rope.k_new = reinterpret_cast<bf16 *>(sc->k_new);
+    qkv.rope.v_new = reinterpret_cast<bf16 *>(sc->v_new);
+    if (s == PHOTON_OK) s = qkv_rope(ctx, qkv, linear_wants_pairs(ctx->clusters, qkv, false), stream);
+    if (s == PHOTON_OK) s = chunk_causal_attn(ctx, chunks, sc->q, unit_ids, sc->att, n, 0, P, scale, P, stream);
     if (s == PHOTON_OK) s = linear(ctx, sc->att, L->wo, L->w_layout, nullptr, U, sc->h, T, D, D, true, stream);
-    if (s == PHOTON_OK) s = photon_rmsnorm(ctx, sc->h, L->g2, L->eps, sc->n, T, D, stream);
+    // the lengths grow behind the attention, with the second normalisation: no kernel of their own between two that wait
+    if (s == PHOTON_OK && launch_rmsnorm(reinterpret_cast<const bf16 *>(sc->h), reinterpret_cast<const bf16 *>(L->g2), L->eps,
+                                         reinterpret_cast<bf16 *>(sc->n), T, D, grow_of(ctx, chunks, unit_ids, n, P),
+                                         static_cast<cudaStream_t>(stream), &ctx->launches) != cudaSuccess)
+        s = PHOTON_ERR_CUDA;
     if (s == PHOTON_OK) s = gate_up(ctx, L, sc, T, stream);
     if (s == PHOTON_OK) s = linear(ctx, sc->act, L->wdown, L->w_layout, nullptr, sc->h, y, T, L->F, D, true, stream);
     return s;

@@ -13,10 +13,11 @@ namespace {
 constexpr int RN_THREADS = 256;
 
 __global__ void __launch_bounds__(RN_THREADS)
-rmsnorm_kernel(const bf16 *x, const bf16 *gamma, float eps, bf16 *out, int cols) {
+rmsnorm_kernel(const bf16 *x, const bf16 *gamma, float eps, bf16 *out, int cols, const Grow g) {
     __shared__ float part[RN_THREADS / 32];
     ptx::grid_dep_wait();                   // x may be the output of the kernel before this one
     ptx::grid_dep_launch();
+    if (g.n) grow_item(g, blockIdx.x * RN_THREADS + threadIdx.x);
     const uint4 *row = reinterpret_cast<const uint4 *>(x + (size_t)blockIdx.x * cols);
     const int n_vec = cols / 8;
     float ss = 0.f;
@@ -60,9 +61,10 @@ rmsnorm_kernel(const bf16 *x, const bf16 *gamma, float eps, bf16 *out, int cols)
 constexpr int RN_MAXV = 8;                  // 16-byte pieces per lane: 32 * 8 * 8 = 2048 columns
 
 __global__ void __launch_bounds__(RN_THREADS)
-rmsnorm_rows_kernel(const bf16 *x, const bf16 *gamma, float eps, bf16 *out, int rows, int cols) {
+rmsnorm_rows_kernel(const bf16 *x, const bf16 *gamma, float eps, bf16 *out, int rows, int cols, const Grow g) {
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
+    if (g.n) grow_item(g, blockIdx.x * RN_THREADS + threadIdx.x);
     const int lane = threadIdx.x & 31;
     const int r = blockIdx.x * (RN_THREADS / 32) + (threadIdx.x >> 5);
     if (r >= rows) return;
@@ -106,15 +108,15 @@ rmsnorm_rows_kernel(const bf16 *x, const bf16 *gamma, float eps, bf16 *out, int 
 
 }  // namespace
 
-cudaError_t launch_rmsnorm(const bf16 *x, const bf16 *gamma, float eps, bf16 *out, int rows, int cols,
+cudaError_t launch_rmsnorm(const bf16 *x, const bf16 *gamma, float eps, bf16 *out, int rows, int cols, const Grow &g,
                            cudaStream_t st, long long *launches) {
     if (rows == 0) return cudaSuccess;
     const int per_cta = RN_THREADS / 32;
     const cudaError_t e =
         cols <= RN_MAXV * 256 && rows >= 1024           // enough rows for a warp per row to fill the GPU
             ? launch_dependent(rmsnorm_rows_kernel, dim3((rows + per_cta - 1) / per_cta), dim3(RN_THREADS), 0, st, 0, x, gamma,
-                               eps, out, rows, cols)
-            : launch_dependent(rmsnorm_kernel, dim3(rows), dim3(RN_THREADS), 0, st, 0, x, gamma, eps, out, cols);
+                               eps, out, rows, cols, g)
+            : launch_dependent(rmsnorm_kernel, dim3(rows), dim3(RN_THREADS), 0, st, 0, x, gamma, eps, out, cols, g);
     ++*launches;
     return e != cudaSuccess ? e : cudaGetLastError();
 }

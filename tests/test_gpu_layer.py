@@ -459,3 +459,90 @@ def test_gate_up_by_pairs_with_features_that_end_inside_a_tile(n, F, out_major):
     silu = gate * torch.sigmoid(gate)
     err = (scratch.tensors["act"].double() - silu * up).abs()
     assert (err <= 2.0 ** -7 * (1.1 * gate.abs() + silu.abs()) * up.abs() + 2.0 ** -8 * (silu * up).abs() + 1e-4).all()
+
+
+def layer_of(g, Hq, Hkv, dh, F, out_major):
+    D = Hq * dh
+
+    def weight(k, m):
+        w = (torch.randn(k, m, generator=g, device="cuda") * k ** -0.5).to(torch.bfloat16)
+        return w.t().contiguous() if out_major else w
+
+    ones = lambda: (1 + 0.1 * torch.randn(D, generator=g, device="cuda")).to(torch.bfloat16)
+    return ph.make_layer(ones(), weight(D, (Hq + 2 * Hkv) * dh), weight(D, D), ones(), weight(D, 2 * F), weight(F, D), int(out_major), F)
+
+
+@pytest.mark.parametrize("Hq,Hkv,dh,P,n", [(4, 2, 64, 4, 3), (4, 2, 64, 4, 700), (8, 8, 128, 8, 5), (8, 8, 128, 8, 40), (8, 8, 128, 8, 200), (16, 4, 128, 3, 100),
+                                           (2, 1, 128, 5, 1000)])
+@pytest.mark.parametrize("out_major", [False, True])
+def test_prefill_rotates_splits_and_appends_in_the_projection(Hq, Hkv, dh, P, n, out_major):
+    """Few rows and many (pairs of CTAs), a head size of either kind, rows that end inside a tile; buffers picked by ids, one without
+    room, one that already holds rows, an id that is not there.  Against the split, the append and the attention called one
+    after the other on the projection the call has left in its scratch: same bits, lengths and status."""
+    cfg = wl.scaled(wl.CONFIGS[4], B=1, Hq=Hq, Hkv=Hkv, dh=dh, D=Hq * dh, P=P, C=P + 1)
+    cap, units, T, scale = 2 * P + 1, n + 2, n * P, dh ** -0.5
+    g = torch.Generator("cuda").manual_seed(n + P)
+    rand = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    layer = layer_of(g, Hq, Hkv, dh, 128, out_major)
+    ids = torch.randperm(units, generator=g, device="cuda").to(torch.int32)[:n].contiguous()
+    len0 = torch.zeros(units, dtype=torch.int32, device="cuda")
+    len0[ids[0].long()] = cap - P + 1                                    # no room for P rows
+    len0[ids[1].long()] = 2
+    ids[2] = units                                                       # no such buffer
+    k0, v0, U = rand(units, Hkv, cap, dh), rand(units, Hkv, cap, dh), rand(n, P, Hq * dh)
+    sc = ph.make_layer_scratch(T, Hq, Hkv, dh, 128, "cuda", torch.bfloat16)
+    with Ctx(cfg, max_queries=T) as c:
+        k, v, ln, y = k0.clone(), v0.clone(), len0.clone(), torch.empty_like(U)
+        ph.photon_decoder_prefill(c.h, layer, sc, U, ph.make_kv(k, v, ln), ids, y, scale=scale)
+        want_status = ph.PHOTON_DEV_CAPACITY | ph.PHOTON_DEV_BAD_INDEX
+        assert c.status() == want_status
+        t = sc.tensors
+        q, kn, vn = torch.empty_like(t["q"]), torch.empty_like(t["k_new"]), torch.empty_like(t["v_new"])
+        pos = torch.arange(P, dtype=torch.int32, device="cuda").repeat(n)
+        ph.photon_rope_split(c.h, t["qkv"], pos, q, kn, vn)
+        for a, b in ((t["q"], q), (t["k_new"], kn), (t["v_new"], vn)):
+            assert np.array_equal(host_bits(a), host_bits(b))
+        k1, v1, ln1 = k0.clone(), v0.clone(), len0.clone()
+        kv1 = ph.make_kv(k1, v1, ln1)
+        ph.photon_kv_append(c.h, kv1, kn.view(n, P, Hkv, dh), vn.view(n, P, Hkv, dh), ids, n, P)
+        att = torch.empty_like(t["att"])
+        ph.photon_chunk_causal_attn(c.h, kv1, q.view(n, P, Hq, dh), ids, att.view(n, P, Hq, dh), n, 0, P, scale)
+        assert c.status() == want_status
+        for a, b in ((k, k1), (v, v1), (t["att"], att)):
+            assert np.array_equal(host_bits(a), host_bits(b))
+        assert torch.equal(ln, ln1)
+
+
+@pytest.mark.parametrize("Hq,Hkv,dh,n", [(4, 2, 64, 5000), (8, 8, 128, 1300), (8, 8, 128, 4100), (2, 1, 128, 9001)])
+@pytest.mark.parametrize("out_major", [False, True])
+def test_decoder_step_of_many_chunks_rotates_and_appends_in_the_projection(Hq, Hkv, dh, n, out_major):
+    """Against the projection, the split, the append and the attention called one after the other: same bits (both projections add the
+    same products in the same order), also for a buffer that is full."""
+    cfg = wl.scaled(wl.CONFIGS[4], B=1, Hq=Hq, Hkv=Hkv, dh=dh, D=Hq * dh, P=4, C=7)
+    cap, F, scale, D = 11, 128, dh ** -0.5, Hq * dh
+    g = torch.Generator("cuda").manual_seed(n)
+    rand = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    layer = layer_of(g, Hq, Hkv, dh, F, out_major)
+    len0 = torch.randint(0, cap + 1, (n,), generator=g, device="cuda", dtype=torch.int32)
+    k0, v0, x = rand(n, Hkv, cap, dh), rand(n, Hkv, cap, dh), rand(n, D)
+    sc = ph.make_layer_scratch(n, Hq, Hkv, dh, F, "cuda", torch.bfloat16)
+    sc.tensors["qkv"].fill_(7.0)
+    with Ctx(cfg, max_queries=n) as c:
+        k, v, ln, y = k0.clone(), v0.clone(), len0.clone(), torch.empty_like(x)
+        ph.photon_decoder_step(c.h, layer, sc, x, ph.make_kv(k, v, ln), y, scale=scale)
+        assert c.status() == ph.PHOTON_DEV_CAPACITY
+        t = sc.tensors
+        assert bool((t["qkv"] == 7.0).all())                             # it took that path
+        g1, wqkv = layer._keep[:2]
+        nx, qkv, q, kn, vn = (torch.empty_like(t[m]) for m in ("n", "qkv", "q", "k_new", "v_new"))
+        ph.photon_rmsnorm(c.h, x, g1, layer.eps, nx)
+        ph.photon_linear(c.h, nx, wqkv, layer.w_layout, None, qkv)
+        ph.photon_rope_split(c.h, qkv, len0, q, kn, vn)
+        k1, v1, ln1, att = k0.clone(), v0.clone(), len0.clone(), torch.empty_like(t["att"])
+        kv1 = ph.make_kv(k1, v1, ln1)
+        ph.photon_kv_append(c.h, kv1, kn, vn)
+        ph.photon_chunk_attn(c.h, kv1, q, None, att, scale=scale)
+        assert c.status() == ph.PHOTON_DEV_CAPACITY
+        for a, b in ((t["q"], q), (k, k1), (v, v1), (t["att"], att)):
+            assert np.array_equal(host_bits(a), host_bits(b))
+        assert torch.equal(ln, ln1)
