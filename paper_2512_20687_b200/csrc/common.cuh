@@ -79,6 +79,7 @@ struct AttnParams {
     int own_rows;            // filled by the launcher: the units' own keys (at most this many rows each) are read by the
                              // shared-prefix kernel, which then writes the final result; 0: a second kernel reads them
     bool over_bus;           // chunk attention: queries and results in host memory
+    bool dependent;          // chunk attention: behind another kernel of the same call
     float scale_log2;        // scale * log2(e): logits are kept in the base-2 domain
     float *partials;
     float *cta_partials;

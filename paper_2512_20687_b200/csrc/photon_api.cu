@@ -40,7 +40,7 @@ int ceil_div(int a, int b) { return (a + b - 1) / b; }
 photon_status attention_common(photon_ctx *ctx, const photon_kv *cache, const photon_bf16 *q,
                                const int32_t *slot, int n_q, photon_bf16 *out, float *lse,
                                float scale, bool chunk, cudaStream_t st, const photon_bf16 *k_new = nullptr,
-                               const photon_bf16 *v_new = nullptr, bool over_bus = false) {
+                               const photon_bf16 *v_new = nullptr, bool over_bus = false, bool dependent = false) {
     if (!ctx) return PHOTON_ERR_INVALID_ARG;
     if (!kv_ok(ctx, cache, !chunk) || (chunk && cache->page_table)) return PHOTON_ERR_INVALID_ARG;
     if (n_q < 0 || (n_q > 0 && (!q || !out))) return PHOTON_ERR_INVALID_ARG;
@@ -83,6 +83,7 @@ photon_status attention_common(photon_ctx *ctx, const photon_kv *cache, const ph
         p.readers = ctx->readers;
     }
     p.over_bus = over_bus;
+    p.dependent = dependent;
     p.max_len = cache->max_len ? cache->max_len : cache->cap;
     p.splits_sh = 0;
     if (!chunk) {
@@ -473,7 +474,8 @@ photon_status layer_step(photon_ctx *ctx, const photon_layer *L, const photon_la
         if (e != cudaSuccess) s = PHOTON_ERR_CUDA;
     }
     if (s == PHOTON_OK)
-        s = local ? photon_chunk_attn(ctx, cache, sc->q, nullptr, sc->att, B, scale, stream)
+        s = local ? attention_common(ctx, cache, sc->q, nullptr, B, sc->att, nullptr, scale, true, static_cast<cudaStream_t>(stream), nullptr,
+                                     nullptr, false, true)
                   : photon_coarse_attn(ctx, cache, sc->q, sc->att, nullptr, scale, stream);
     if (s == PHOTON_OK) s = linear(ctx, sc->att, L->wo, L->w_layout, nullptr, x, sc->h, B, D, D, true, stream);
     if (s == PHOTON_OK) s = photon_rmsnorm(ctx, sc->h, L->g2, L->eps, sc->n, B, D, stream);
