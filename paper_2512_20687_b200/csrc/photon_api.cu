@@ -598,9 +598,16 @@ photon_status step_impl(photon_ctx *ctx, const photon_step_args *a, photon_strea
     // built, sit between the converter's output and the chunk caches): it runs beside them on a
     // low-priority stream that forks from `stream` here and joins it again before the call returns, so
     // for the caller the whole step is still ordered on `stream`.  Large chunk workloads stay in line:
-    // two kernels that are both bound by HBM gain nothing from running side by side.
-    const bool beside = a->Nc > 0 &&
-                        (size_t)a->Nc * c.Hkv * a->chunks->cap * c.dh * 4 <= (size_t(32) << 20);
+    // two kernels that are both bound by HBM gain nothing from running side by side.  So do steps of at most 8 MB that are launched
+    // one by one: the device is through with all three kernels before the host has enqueued them (9 of 20 us), and the fork and the
+    // join are four calls more (2 sequences of the 256-wide model, 8 chunks each, 20.3 -> 18.7 us; replayed they would cost 1.5).
+    const size_t chunk_bytes = a->Nc > 0 ? (size_t)a->Nc * c.Hkv * a->chunks->cap * c.dh * 4 : 0;
+    const size_t step_bytes = chunk_bytes + (size_t)c.D * c.P * c.D * 2 +
+                              (size_t)a->coarse->n_units * c.Hkv * (a->coarse->max_len ? a->coarse->max_len : a->coarse->cap) * c.dh * 4;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) return PHOTON_ERR_CUDA;
+    const bool tiny = !hp && capture == cudaStreamCaptureStatusNone && step_bytes <= (size_t(8) << 20);
+    const bool beside = a->Nc > 0 && chunk_bytes <= (size_t(32) << 20) && !tiny;
     photon_status s = PHOTON_OK;
     // With host buffers and a declared split the two halves of either buffer travel apart.  Where both host buffers are
     // mapped into the device and the chunk attention's arrays lie wholly in its halves of the staging areas, that
@@ -675,8 +682,6 @@ photon_status step_impl(photon_ctx *ctx, const photon_step_args *a, photon_strea
     // way.  In a captured step both start at the same time, and where the chunk attention is the first node its CTAs take
     // registers from the coarse attention's first wave: there it follows (replayed, 64 sequences 25.2 -> 23.6 us, 16 long ones
     // 60.1 -> 57.9, 77 ragged paged ones 40.3 -> 37.0; called one by one that order is no faster, the long ones 59.8 and 60.5).
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (beside && cudaStreamIsCapturing(st, &capture) != cudaSuccess) s = PHOTON_ERR_CUDA;
     const bool chunks_first = capture == cudaStreamCaptureStatusNone;
     if (beside && (chunks_first || s != PHOTON_OK) && chunks_beside() != PHOTON_OK) return s;
     // The append is one row per unit, in place: for a batch whose lengths fit the attention kernel's shared memory it
@@ -716,7 +721,7 @@ photon_status step_impl(photon_ctx *ctx, const photon_step_args *a, photon_strea
         if (cudaStreamWaitEvent(st, ctx->ev_join, 0) != cudaSuccess && s == PHOTON_OK) s = PHOTON_ERR_CUDA;
     } else if (s == PHOTON_OK && a->Nc > 0) {
         s = attention_common(ctx, a->chunks, q_chunk, slot, a->Nc, out_chunk, nullptr, a->scale_chunk, true, st, nullptr, nullptr,
-                             direct);
+                             direct, tiny);
     }
     if (copying && cudaStreamWaitEvent(st, ctx->ev_copy, 0) != cudaSuccess && s == PHOTON_OK) s = PHOTON_ERR_CUDA;
     if (s == PHOTON_OK && hp && !copy_out(hp, copying ? early_end : 0, apart || direct ? hp->out_split : hp->out_bytes, st))
