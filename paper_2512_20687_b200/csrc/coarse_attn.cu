@@ -50,8 +50,10 @@ constexpr int CTAS_PER_SM = 2;
 // others.  77 sequences of 0 to 1000 rows, 16/4 heads: 21.7 us with streams of up to 8 tiles whole, 18.6 with 16; longer limits
 // leave long caches to too few CTAs (20 of 0 to 3000 rows: 18.5, and 20.1 with 24 tiles whole).  Boundaries close to an end of a
 // longer stream move there: 130 of 0 to 2000 rows 50.3 -> 49.7 us; with 4 and 8 tiles instead of 2, 20 x 3000 is slower (18.8, 19.3).
-constexpr int SNAP = 16;                   // streams of at most this many tiles are never cut
-constexpr int EDGE = 2;                    // others not within this many tiles of an end
+// With less than four tiles per CTA the length of the longest share counts, and streams are cut as soon as they exceed 8 tiles.
+constexpr int SNAP = 16, SNAP_THIN = 8;    // streams of at most this many tiles are never cut
+constexpr int EDGE = 2, EDGE_THIN = 0;     // others not within this many tiles of an end
+constexpr int THIN = 4;
 static_assert(2 * EDGE <= SNAP, "a boundary cannot be close to both ends of a stream that is cut");
 constexpr int NLEN = 768;                  // lengths of the first NLEN units are kept in shared memory
 
@@ -126,6 +128,7 @@ struct Share {
     int n_cta;               // CTAs that take part
     long long t0, t1;        // this CTA's tiles [t0, t1)
     int u0, rem;             // tile t0 is tile `rem` of the Hkv * nt tiles of unit u0
+    int edge;                // EDGE or EDGE_THIN
 };
 
 // Position in the sequence of tiles: tile j of the stream (unit u, KV head h).  The lengths of units
@@ -343,7 +346,7 @@ __device__ __forceinline__ void process_block(uint32_t kt, uint32_t vt, int kb, 
 // The even deal of the tile sequence over the grid, found by all threads of the CTA from len[]: every
 // length is read once (and left in shared memory for units below NLEN), a block-wide prefix sum of tile
 // counts follows, then the two boundaries of this CTA's share.  Boundary c is tile T*c/n_cta; where it
-// falls inside a short stream (<= SNAP tiles) it moves to the nearer end of that stream, and where it falls
+// falls inside a short stream (at most SNAP tiles, or SNAP_THIN) it moves to the nearer end of that stream, and where it falls
 // within EDGE tiles of an end of a longer one to that end.  Where all units have as many tiles, only as many CTAs
 // take part as share the streams out evenly (ctas_equal).  sc: [0..5] warp sums, [8] u0, [9] rem, [12] t0, [14] t1.
 template <bool PAGED>
@@ -393,6 +396,9 @@ __device__ __forceinline__ Share deal(const AttnParams &p, int *sc, int *slen, i
     // every CTA that takes part owns at least one tile of the even deal, so the CTAs holding a cut stream
     // are consecutive
     sh.n_cta = (int)min((long long)(same ? min(p.ctas_equal, (int)gridDim.x) : gridDim.x), sh.T);
+    const bool thin = sh.T < (long long)THIN * sh.n_cta;
+    const int snap = thin ? SNAP_THIN : SNAP;
+    sh.edge = thin ? EDGE_THIN : EDGE;
     {
         const long long lo = (long long)(before + incl - mine) * p.Hkv, hi = lo + (long long)mine * p.Hkv;
 #pragma unroll
@@ -411,8 +417,8 @@ __device__ __forceinline__ Share deal(const AttnParams &p, int *sc, int *slen, i
                     int rem = (int)(x - pre), uu = u;
                     const int j = rem % nt;
                     long long bx = x;
-                    if (j != 0 && (nt <= SNAP ? 2 * j <= nt : j <= EDGE)) { bx = x - j; rem -= j; }
-                    else if (j != 0 && (nt <= SNAP || nt - j <= EDGE)) { bx = x + (nt - j); rem += nt - j; }
+                    if (j != 0 && (nt <= snap ? 2 * j <= nt : j <= sh.edge)) { bx = x - j; rem -= j; }
+                    else if (j != 0 && (nt <= snap || nt - j <= sh.edge)) { bx = x + (nt - j); rem += nt - j; }
                     if (rem == nt * p.Hkv) {                      // moved to the start of the next unit that has keys
                         rem = 0;
                         do { ++uu; } while (uu < p.n_units && len_of(uu) == 0);
@@ -896,8 +902,8 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
                 if (!whole) {
                     // CTAs that hold a piece of this stream: first and last
                     const long long te = seg_t + w.nt;
-                    meta[3] = (int)(((seg_t + EDGE + 1) * n_cta - 1) / T);     // (boundaries within EDGE tiles of an end have moved there)
-                    meta[4] = (int)(((te - EDGE) * n_cta - 1) / T);
+                    meta[3] = (int)(((seg_t + sh.edge + 1) * n_cta - 1) / T);  // (boundaries within that many tiles of an end have moved there)
+                    meta[4] = (int)(((te - sh.edge) * n_cta - 1) / T);
                 }
             }
             if (direct) ptx::named_bar_sync(1, NW * 32);
