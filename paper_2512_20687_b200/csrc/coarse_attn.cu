@@ -30,6 +30,7 @@
 // result does not depend on arrival order.  Partials of a shared prefix, when
 // present, were produced by an earlier launch and are folded in at the same
 // point.
+#include <limits.h>
 #include <math_constants.h>
 
 #include "common.cuh"
@@ -56,6 +57,7 @@ constexpr int EDGE = 2, EDGE_THIN = 0;     // others not within this many tiles 
 constexpr int THIN = 4;
 static_assert(2 * EDGE <= SNAP, "a boundary cannot be close to both ends of a stream that is cut");
 constexpr int NLEN = 768;                  // lengths of the first NLEN units are kept in shared memory
+constexpr int SCALARS = 48;                // words of shared memory between the barriers and those lengths
 
 template <int DH>
 struct Ring {
@@ -69,7 +71,7 @@ __host__ __device__ inline int q_slot_bytes(int G, int dh) { return (G * dh * 2 
 template <int DH>
 size_t smem_bytes(int G) {
     return size_t(STAGES) * (Ring<DH>::STAGE_BYTES + q_slot_bytes(G, DH) + 2 * DH * 2 /*a new K and V row*/) +
-           size_t(NW) * G * (DH + 2) * sizeof(float) + 128 /*barriers*/ + 128 /*scalars*/ + NLEN * sizeof(int);
+           size_t(NW) * G * (DH + 2) * sizeof(float) + 128 /*barriers*/ + SCALARS * sizeof(int) + NLEN * sizeof(int);
 }
 
 __device__ __forceinline__ int tiles_of(int len) { return (len + BN - 1) / BN; }
@@ -348,49 +350,52 @@ __device__ __forceinline__ void process_block(uint32_t kt, uint32_t vt, int kb, 
 // counts follows, then the two boundaries of this CTA's share.  Boundary c is tile T*c/n_cta; where it
 // falls inside a short stream (at most SNAP tiles, or SNAP_THIN) it moves to the nearer end of that stream, and where it falls
 // within EDGE tiles of an end of a longer one to that end.  Where all units have as many tiles, only as many CTAs
-// take part as share the streams out evenly (ctas_equal).  sc: [0..5] warp sums, [8] u0, [9] rem, [12] t0, [14] t1.
+// take part as share the streams out evenly (ctas_equal).  sc: [0..5] warp sums, [8] u0, [9] rem, [12] t0, [14] t1, [32..43] fewest and
+// most tiles of a unit, by warp.  The deal is a function of the tile counts of the lengths in slen and of nothing else (units from NLEN on
+// have no copy there and are dealt after the dependency wait): a length is read once, and what is compared with it later is that copy.
 template <bool PAGED>
 __device__ __forceinline__ Share deal(const AttnParams &p, int *sc, int *slen, int cta) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     auto len_of = [&](int u) { return eff_len(p, u < NLEN ? slen[u] : ld_len<PAGED>(p, u)); };
     const int per = (p.n_units + THREADS - 1) / THREADS;
     const int ub = min(p.n_units, (int)threadIdx.x * per), ue = min(p.n_units, ub + per);
-    int mine = 0;
-    bool same = true;                                             // as many tiles in every unit
+    int mine = 0, fewest = INT_MAX, most = -1;                    // tiles of this thread's units; of one of them
     if (per <= LPT) {                                             // all loads in flight together
         int len[LPT];
-        const int first = ld_len<PAGED>(p, 0);
         load_lengths<PAGED>(p, ub, ue, len, nullptr);
-        const int nt0 = tiles_of(eff_len(p, first));
 #pragma unroll
         for (int i = 0; i < LPT; ++i)
             if (ub + i < ue) {
                 const int nt = tiles_of(eff_len(p, len[i]));
-                slen[ub + i] = len[i]; mine += nt; same &= nt == nt0;
+                slen[ub + i] = len[i]; mine += nt; fewest = min(fewest, nt); most = max(most, nt);
             }
     } else {
-        const int nt0 = tiles_of(eff_len(p, ld_len<PAGED>(p, 0)));
         for (int u = ub; u < ue; ++u) {
             const int len = ld_len<PAGED>(p, u);
             if (u < NLEN) slen[u] = len;
             const int nt = tiles_of(eff_len(p, len));
-            mine += nt; same &= nt == nt0;
+            mine += nt; fewest = min(fewest, nt); most = max(most, nt);
         }
     }
+    fewest = __reduce_min_sync(0xffffffffu, fewest);
+    most = __reduce_max_sync(0xffffffffu, most);
     int incl = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int v = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += v;
     }
-    if (lane == 31) sc[warp] = incl;
-    same = __syncthreads_and(same);
+    int2 *extent = reinterpret_cast<int2 *>(sc + 32);
+    if (lane == 31) { sc[warp] = incl; extent[warp] = make_int2(fewest, most); }
+    __syncthreads();
     int before = 0, all = 0;
 #pragma unroll
     for (int w = 0; w < THREADS / 32; ++w) {
         if (w < warp) before += sc[w];
         all += sc[w];
+        fewest = min(fewest, extent[w].x); most = max(most, extent[w].y);
     }
+    const bool same = fewest == most;                             // as many tiles in every unit
     Share sh;
     sh.T = (long long)all * p.Hkv;
     // every CTA that takes part owns at least one tile of the even deal, so the CTAs holding a cut stream
@@ -473,7 +478,7 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
     volatile int *dead = sc + 11;                               // [16..23] description of the stream in `red`
     volatile int *meta = sc + 16;
     volatile int *tile_at = sc + 24;                            // [STAGES] first cache row of the tile in a stage
-    int *slen = sc + 32;                                        // [NLEN] lengths of the first units
+    int *slen = sc + SCALARS;                                   // [NLEN] lengths of the first units
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cta = blockIdx.x;
@@ -497,8 +502,8 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
 
     // ---- the deal, ahead of the kernel before this one.  The lengths as they read now may still change
     // (an append in flight), and no key or value is touched yet; after the dependency wait every length is
-    // read again, and the deal stands if no unit's tile count differs (it depends on nothing else), so
-    // that one trip to the L2 and one barrier are all that separates the wait from the first load.
+    // read again, and the deal stands if no unit's tile count differs from that of the length it was made of (slen; it depends
+    // on nothing else), so that one trip to the L2 and one barrier are all that separates the wait from the first load.
     // Batches beyond NLEN units keep no copy to compare with and deal after the wait.
     const bool ahead = p.n_units <= NLEN;
     Share sh;

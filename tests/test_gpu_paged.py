@@ -192,3 +192,63 @@ def test_streams_at_the_edges_of_the_deal(n, S, lengths, paged):
     want_lse = torch.logsumexp(logit, -1).view(n, Hq)
     fin = torch.isfinite(want_lse)
     assert torch.equal(torch.isneginf(lse), ~fin) and (lse.double() - want_lse)[fin].abs().max() < 2e-3
+
+
+# tile counts of the units before the append and after it: equal and all open a tile (one, two, eighteen tiles: streams that are cut);
+# equal and none does; equal only before; equal only after
+BEHIND_AN_APPEND = [(64,), (128,), (1088,), (127,), (0,), (63, 64), (1087, 1088), (64, 65), (1089, 1088)]
+
+
+@pytest.mark.parametrize("lengths", BEHIND_AN_APPEND)
+@pytest.mark.parametrize("n", [77, 80])
+@pytest.mark.parametrize("paged", [False, True])
+def test_deal_of_more_streams_than_ctas_behind_an_append(n, lengths, paged):
+    """More streams than CTAs: how many CTAs take part depends on whether the tile counts are equal, and the attention deals while
+    the append in front of it writes the lengths.  Behind reads of varied length (the probe), so that its CTAs meet the append at
+    different points: the bits of a call on an idle device each time, also of a second attention (tickets and counters are
+    as they should be), status clear, and the result within its two roundings to bf16 of torch in 64 bits: the output's (2^-8 of the
+    value) and the weights' (2^-8 of the weighted sum of the absolute values)."""
+    Hq, Hkv, dh, S = 8, 4, 64, 64 * (max(lengths) // 64 + 1)
+    cfg = wl.scaled(wl.CONFIGS[1], B=n, Hq=Hq, Hkv=Hkv, dh=dh, D=Hq * dh)
+    g = torch.Generator("cuda").manual_seed(n + len(lengths) + S)
+    rand = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    len0 = dev_i32([lengths[u % len(lengths)] for u in range(n)])
+    k, v, q, k_new, v_new = rand(n, Hkv, S, dh), rand(n, Hkv, S, dh), rand(n, Hq, dh), rand(n, Hkv, dh), rand(n, Hkv, dh)
+    ln, ppu = len0.clone(), S // 64
+    at = torch.arange(n, device="cuda")
+    want_k, want_v = k.double(), v.double()
+    want_k[at, :, len0.long()], want_v[at, :, len0.long()] = k_new.double(), v_new.double()
+    if paged:
+        order = torch.randperm(n * ppu, generator=g, device="cuda")
+        cut = lambda t: t.view(n, Hkv, ppu, 64, dh).transpose(1, 2).reshape(n * ppu, Hkv, 64, dh)
+        pk, pv = torch.empty_like(cut(k)), torch.empty_like(cut(v))
+        pk[order], pv[order] = cut(k), cut(v)
+        kv = ph.make_kv(pk, pv, ln, page_table=order.to(torch.int32).view(n, ppu).contiguous())
+    else:
+        kv = ph.make_kv(k, v, ln)
+    held = torch.empty(64 << 20, dtype=torch.uint8, device="cuda").random_()
+    scale, first = dh ** -0.5, None
+    with Ctx(cfg) as c:
+        for turn in range(60):
+            outs = [(torch.empty_like(q), torch.empty(n, Hq, device="cuda")) for _ in range(2)]
+            ln.copy_(len0)
+            torch.cuda.synchronize()
+            if turn:
+                ph.photon_read_probe(c.h, held[:(turn * 1237 % 4096) * 16384])      # 0 to 64 MB
+            ph.photon_kv_append(c.h, kv, k_new, v_new)
+            if not turn:
+                torch.cuda.synchronize()
+            for out, lse in outs:
+                ph.photon_coarse_attn(c.h, kv, q, out, lse, scale)
+            assert c.status() == 0
+            got = [torch.cat([out.view(torch.int16).int().view(n, -1), lse.view(torch.int32)], 1) for out, lse in outs]
+            first = got[0] if first is None else first
+            assert torch.equal(got[0], first) and torch.equal(got[1], first), turn
+            assert torch.equal(ln, len0 + 1)
+    out, lse = outs[0]
+    logit = torch.einsum("nhgd,nhsd->nhgs", q.double().view(n, Hkv, Hq // Hkv, dh), want_k) * scale
+    logit.masked_fill_((torch.arange(S, device="cuda") > len0[:, None])[:, None, None], float("-inf"))
+    w = torch.softmax(logit, -1)
+    want, size = (torch.einsum("nhgs,nhsd->nhgd", w, x).reshape(n, Hq, dh) for x in (want_v, want_v.abs()))
+    assert ((out.double() - want).abs() <= 2.0 ** -8 * (want.abs() + size) + 1e-5).all()
+    assert (lse.double() - torch.logsumexp(logit, -1).view(n, Hq)).abs().max() < 2e-3
