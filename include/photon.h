@@ -220,7 +220,9 @@ photon_status photon_linear(photon_ctx *ctx, const photon_bf16 *x, const photon_
  * weights in the order w_layout names: wqkv [D, (Hq + 2 Hkv) dh], wo [Hq dh,
  * D], wgu [D, 2F], wdown [F, D]; g1, g2 [D].  F a multiple of 64.  The
  * caller owns the intermediates in `scratch` (sizes beside the fields); each
- * is rounded to bf16 where the next kernel reads it.  y may alias x.  Where
+ * is rounded to bf16 where the next kernel reads it.  y may alias x, and q,
+ * act and (prefill) k_new and v_new may lie over n, which is through by then;
+ * kernels that would join them then run one after the other.  Where
  * the gate/up projection's slabs of 64 features occupy at least half of the
  * GPU's SMs (F / 64 slabs per 128 rows), and with many rows, that
  * projection and the activation are one launch and scratch->gu is left

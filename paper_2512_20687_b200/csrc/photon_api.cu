@@ -374,9 +374,17 @@ photon_status photon_swiglu(photon_ctx *ctx, const photon_bf16 *gu, photon_bf16 
 }
 
 namespace {
+// Whether the arrays share memory.  A caller may lay arrays of the scratch over one another where one is through before the next is
+// written; a kernel that does several kernels' work writes its results while others of its CTAs still read its input, so where those
+// two share memory the kernels run one after the other.
+bool overlap(const photon_bf16 *a, size_t na, const photon_bf16 *b, size_t nb) {
+    const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
+    return pa < pb + nb * sizeof(photon_bf16) && pb < pa + na * sizeof(photon_bf16);
+}
+
 // gate/up projection and activation: act [rows, F] = silu(n Wg) * (n Wu).  One fused launch (gu is then not written)
 // of the kernel of CTA pairs with many rows, of the slab kernel where 64-feature slabs occupy most of the GPU;
-// else the projection followed by photon_swiglu.
+// else, or where act lies over n, the projection followed by photon_swiglu.
 photon_status gate_up(photon_ctx *ctx, const photon_layer *L, const photon_layer_scratch *sc, int rows,
                       photon_stream stream) {
     const photon_config &c = ctx->cfg;
@@ -388,11 +396,12 @@ photon_status gate_up(photon_ctx *ctx, const photon_layer *L, const photon_layer
     p.w_out_major = (L->w_layout == PHOTON_W_OUT_MAJOR);
     p.w_ahead = true;
     p.status = ctx->status;
-    if (linear_wants_pairs(ctx->clusters, p, true)) {
+    const bool apart = !overlap(sc->act, (size_t)rows * L->F, sc->n, (size_t)rows * c.D);
+    if (apart && linear_wants_pairs(ctx->clusters, p, true)) {
         const cudaError_t e = launch_gate_up_pairs(ctx, p, static_cast<cudaStream_t>(stream), &ctx->launches);
         return e == cudaSuccess ? PHOTON_OK : PHOTON_ERR_CUDA;
     }
-    if (gate_up_fits_small_tiles(ctx, p)) {                                // one launch, gu is not written
+    if (apart && gate_up_fits_small_tiles(ctx, p)) {                                // one launch, gu is not written
         const cudaError_t e = launch_gate_up(ctx, p, static_cast<cudaStream_t>(stream), &ctx->launches);
         return e == cudaSuccess ? PHOTON_OK : PHOTON_ERR_CUDA;
     }
@@ -456,7 +465,7 @@ photon_status layer_step(photon_ctx *ctx, const photon_layer *L, const photon_la
     // back with 16384 chunks of width 1024) is not written: projection and split 127 us, 75 so.  Few: a cut into whole heads costs
     // the small kernel about as much as the split kernel.
     const ConvParams qkv = qkv_rope_params(ctx, L, sc, B, cache, nullptr, 0);
-    const bool fused = local && linear_wants_pairs(ctx->clusters, qkv, false);
+    const bool fused = local && linear_wants_pairs(ctx->clusters, qkv, false) && !overlap(sc->q, (size_t)B * D, sc->n, (size_t)B * D);
     if (fused) {
         if (s == PHOTON_OK) s = qkv_rope(ctx, qkv, true, stream);
         if (s == PHOTON_OK && launch_grow(grow_of(ctx, cache, nullptr, B, 1), static_cast<cudaStream_t>(stream), &ctx->launches) != cudaSuccess)
@@ -512,16 +521,28 @@ photon_status photon_decoder_prefill(photon_ctx *ctx, const photon_layer *L, con
     photon_status s = photon_rmsnorm(ctx, U, L->g1, L->eps, sc->n, T, D, stream);
     // one projection that rotates, splits and appends, instead of three kernels (a trip between kernels each; 64 chunks of 4 rows, 2048
     // wide, 64.4 -> 62.2 us, 200 of 8 rows, 1024 wide, 88.6 -> 78.2); the intermediates are written all the same
-    ConvParams qkv = qkv_rope_params(ctx, L, sc, T, chunks, unit_ids, P);
-    qkv.rope.qkv = reinterpret_cast<bf16 *>(sc->qkv);
-    qkv.rope.k_new = reinterpret_cast<bf16 *>(sc->k_new);
-    qkv.rope.v_new = reinterpret_cast<bf16 *>(sc->v_new);
-    if (s == PHOTON_OK) s = qkv_rope(ctx, qkv, linear_wants_pairs(ctx->clusters, qkv, false), stream);
-    if (s == PHOTON_OK) s = chunk_causal_attn(ctx, chunks, sc->q, unit_ids, sc->att, n, 0, P, scale, P, stream);
+    const size_t in = (size_t)T * D, kv = (size_t)T * c.Hkv * c.dh;
+    const bool fused = !overlap(sc->q, in, sc->n, in) && !overlap(sc->k_new, kv, sc->n, in) && !overlap(sc->v_new, kv, sc->n, in);
+    if (fused) {
+        ConvParams qkv = qkv_rope_params(ctx, L, sc, T, chunks, unit_ids, P);
+        qkv.rope.qkv = reinterpret_cast<bf16 *>(sc->qkv);
+        qkv.rope.k_new = reinterpret_cast<bf16 *>(sc->k_new);
+        qkv.rope.v_new = reinterpret_cast<bf16 *>(sc->v_new);
+        if (s == PHOTON_OK) s = qkv_rope(ctx, qkv, linear_wants_pairs(ctx->clusters, qkv, false), stream);
+    } else {
+        if (s == PHOTON_OK) s = linear(ctx, sc->n, L->wqkv, L->w_layout, nullptr, nullptr, sc->qkv, T, D, (c.Hq + 2 * c.Hkv) * c.dh, true, stream);
+        if (s == PHOTON_OK &&
+            launch_rope_split(reinterpret_cast<const bf16 *>(sc->qkv), nullptr, P, T, c.Hq, c.Hkv, c.dh, L->theta,
+                              reinterpret_cast<bf16 *>(sc->q), reinterpret_cast<bf16 *>(sc->k_new), reinterpret_cast<bf16 *>(sc->v_new),
+                              static_cast<cudaStream_t>(stream), &ctx->launches) != cudaSuccess)
+            s = PHOTON_ERR_CUDA;
+        if (s == PHOTON_OK) s = photon_kv_append(ctx, chunks, sc->k_new, sc->v_new, unit_ids, n, P, stream);
+    }
+    if (s == PHOTON_OK) s = chunk_causal_attn(ctx, chunks, sc->q, unit_ids, sc->att, n, 0, P, scale, fused ? P : 0, stream);
     if (s == PHOTON_OK) s = linear(ctx, sc->att, L->wo, L->w_layout, nullptr, U, sc->h, T, D, D, true, stream);
     // the lengths grow behind the attention, with the second normalisation: no kernel of their own between two that wait
     if (s == PHOTON_OK && launch_rmsnorm(reinterpret_cast<const bf16 *>(sc->h), reinterpret_cast<const bf16 *>(L->g2), L->eps,
-                                         reinterpret_cast<bf16 *>(sc->n), T, D, grow_of(ctx, chunks, unit_ids, n, P),
+                                         reinterpret_cast<bf16 *>(sc->n), T, D, fused ? grow_of(ctx, chunks, unit_ids, n, P) : Grow{},
                                          static_cast<cudaStream_t>(stream), &ctx->launches) != cudaSuccess)
         s = PHOTON_ERR_CUDA;
     if (s == PHOTON_OK) s = gate_up(ctx, L, sc, T, stream);

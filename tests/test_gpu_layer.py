@@ -546,3 +546,65 @@ def test_decoder_step_of_many_chunks_rotates_and_appends_in_the_projection(Hq, H
         for a, b in ((t["q"], q), (k, k1), (v, v1), (t["att"], att)):
             assert np.array_equal(host_bits(a), host_bits(b))
         assert torch.equal(ln, ln1)
+
+
+def assert_same_but_for_roundings(got, want):
+    """Sums in another order can round differently to bf16 in every array on the way (nine, 2^-8 of a value each, on either side: 0.07
+    of values that reach twice the size of the result's); rows of another array in the place of n are off by more than the result."""
+    for a, b in zip(got, want):
+        a, b = a.double(), b.double()
+        assert ((a - b).abs() <= 2.0 ** -3 * b.abs().clamp(min=float(b.square().mean().sqrt()))).all()
+
+
+def lay_over(sc, name):
+    """The scratch with one of its arrays at the place of `n` (which is made as large as both)."""
+    t = sc.tensors
+    room = torch.empty(max(t["n"].numel(), t[name].numel()), dtype=torch.bfloat16, device="cuda")
+    for m in ("n", name):
+        t[m] = room[:t[m].numel()].view(t[m].shape)
+        setattr(sc, m, t[m].data_ptr())
+    return sc
+
+
+@pytest.mark.parametrize("name", ["q", "act", "k_new", "v_new"])
+@pytest.mark.parametrize("Hq,Hkv,dh,F,n", [(4, 2, 64, 1088, 40), (8, 8, 128, 1088, 300), (8, 8, 128, 2816, 1300)])
+def test_prefill_with_scratch_arrays_over_the_normalised_rows(name, Hq, Hkv, dh, F, n):
+    """n is through when q, k_new, v_new and act are written: they may lie over it."""
+    P = 4
+    cfg = wl.scaled(wl.CONFIGS[4], B=1, Hq=Hq, Hkv=Hkv, dh=dh, D=Hq * dh, P=P, C=3)
+    g = torch.Generator("cuda").manual_seed(n + F)
+    rand = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    layer, U = layer_of(g, Hq, Hkv, dh, F, True), rand(n, P, Hq * dh)
+    k0, v0, got = rand(n, Hkv, 7, dh), rand(n, Hkv, 7, dh), []
+    with Ctx(cfg, max_queries=n * P) as c:
+        for over in (False, True):
+            sc = ph.make_layer_scratch(n * P, Hq, Hkv, dh, F, "cuda", torch.bfloat16)
+            if over:
+                lay_over(sc, name)
+            k, v, ln, y = k0.clone(), v0.clone(), torch.zeros(n, dtype=torch.int32, device="cuda"), torch.empty_like(U)
+            ph.photon_decoder_prefill(c.h, layer, sc, U, ph.make_kv(k, v, ln), None, y, scale=dh ** -0.5)
+            assert c.status() == 0 and bool((ln == P).all())
+            got.append([y, k, v])
+    assert_same_but_for_roundings(*got)
+
+
+@pytest.mark.parametrize("name", ["q", "act"])
+@pytest.mark.parametrize("Hq,Hkv,dh,F,n", [(4, 2, 64, 1088, 300), (8, 8, 128, 1088, 1601), (8, 8, 128, 2816, 5000)])
+def test_decoder_step_with_scratch_arrays_over_the_normalised_rows(name, Hq, Hkv, dh, F, n):
+    """As above, for one row per chunk."""
+    cfg = wl.scaled(wl.CONFIGS[4], B=1, Hq=Hq, Hkv=Hkv, dh=dh, D=Hq * dh, P=4, C=7)
+    g = torch.Generator("cuda").manual_seed(n + F)
+    rand = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    layer, x = layer_of(g, Hq, Hkv, dh, F, True), rand(n, Hq * dh)
+    len0 = torch.randint(0, 11, (n,), generator=g, device="cuda", dtype=torch.int32)
+    k0, v0, got = rand(n, Hkv, 11, dh), rand(n, Hkv, 11, dh), []
+    with Ctx(cfg, max_queries=n) as c:
+        for over in (False, True):
+            sc = ph.make_layer_scratch(n, Hq, Hkv, dh, F, "cuda", torch.bfloat16)
+            if over:
+                lay_over(sc, name)
+            k, v, ln, y = k0.clone(), v0.clone(), len0.clone(), torch.empty_like(x)
+            ph.photon_decoder_step(c.h, layer, sc, x, ph.make_kv(k, v, ln), y, scale=dh ** -0.5)
+            assert c.status() == 0 and torch.equal(ln, len0 + 1)
+            got.append([y, k, v])
+    assert_same_but_for_roundings(*got)
