@@ -30,7 +30,6 @@
 // result does not depend on arrival order.  Partials of a shared prefix, when
 // present, were produced by an earlier launch and are folded in at the same
 // point.
-#include <limits.h>
 #include <math_constants.h>
 
 #include "common.cuh"
@@ -46,18 +45,25 @@ constexpr int STAGES = 3;
 constexpr int HALF_BYTES = BN * 128;       // 64 rows x 64 elements, swizzled
 constexpr int BOX_BYTES = BOX * 128;
 constexpr int CTAS_PER_SM = 2;
-// Where a stream may be cut.  A cut costs 3 to 5 us at the end of a CTA (the part's stores, a fence, a ticket and the merge, a trip
-// to the L2 each); a share that is some tiles longer costs little, because the CTAs that are through leave their bandwidth to the
-// others.  77 sequences of 0 to 1000 rows, 16/4 heads: 21.7 us with streams of up to 8 tiles whole, 18.6 with 16; longer limits
-// leave long caches to too few CTAs (20 of 0 to 3000 rows: 18.5, and 20.1 with 24 tiles whole).  Boundaries close to an end of a
-// longer stream move there: 130 of 0 to 2000 rows 50.3 -> 49.7 us; with 4 and 8 tiles instead of 2, 20 x 3000 is slower (18.8, 19.3).
-// With less than four tiles per CTA the length of the longest share counts, and streams are cut as soon as they exceed 8 tiles.
-constexpr int SNAP = 16, SNAP_THIN = 8;    // streams of at most this many tiles are never cut
-constexpr int EDGE = 2, EDGE_THIN = 0;     // others not within this many tiles of an end
-constexpr int THIN = 4;
-static_assert(2 * EDGE <= SNAP, "a boundary cannot be close to both ends of a stream that is cut");
+// Where a stream may be cut.  Streams of at most 8 tiles never are.  What a cut costs at the end of a CTA (the part's stores, a fence, a
+// ticket and the merge, a trip to the L2 each) depends on the size of a part, G query heads of DH floats: 1 us with 2 heads of 64 features
+// or one of 128, 4 with 4 of 128, 12 with 16 of 128; a tile takes 0.4 to 0.7.  So only with 4 heads of 128 and more do longer streams stay
+// whole, up to 16 tiles:
+//  - with equal lengths where the longest share is then at most 5 tiles longer than the even one (whole_equal; with 8 heads and more where a
+//    stream would be cut in two): 128 streams of 9 or 10 tiles 12.8 and 13.4 us in halves, 11.0 and 11.7 whole, 96 of 16 14.6 and 15.4,
+//    64 of 16 in four parts each 12.2 and 15.3;
+//  - with different lengths, 4 heads and 4 to 10 tiles per CTA (below, the length of the longest share is what counts), streams of at most 7 tiles more than the even share that are not close to
+//    it (a CTA gets two of those or none; 300 of 11 to 13 tiles, even share 12.5: 25.1 and 27.8 us); boundaries within 2 tiles of an end of
+//    another stream move there.  75 sequences of 0 to 1000 rows 20.6 -> 18.1 us, 32 of 0 to 1800 18.9 -> 16.9;
+//  - with different lengths and 8 heads or more, streams that are much longer or much shorter than the even share; ends likewise.
+template <int DH, int GP>
+struct Cuts {
+    static constexpr bool DEAR = DH == 128 && GP >= 4, VERY_DEAR = DH == 128 && GP >= 8;
+    static constexpr int WHOLE = 8, WHOLE_DEAR = 16, THIN = 4, THICK = 10, EDGE = 2;
+    static_assert(2 * EDGE <= WHOLE, "a boundary cannot be close to both ends of a stream that is cut");
+};
 constexpr int NLEN = 768;                  // lengths of the first NLEN units are kept in shared memory
-constexpr int SCALARS = 48;                // words of shared memory between the barriers and those lengths
+constexpr int SCALARS = 40;                // words of shared memory between the barriers and those lengths
 
 template <int DH>
 struct Ring {
@@ -130,7 +136,7 @@ struct Share {
     int n_cta;               // CTAs that take part
     long long t0, t1;        // this CTA's tiles [t0, t1)
     int u0, rem;             // tile t0 is tile `rem` of the Hkv * nt tiles of unit u0
-    int edge;                // EDGE or EDGE_THIN
+    int edge;                // boundaries within so many tiles of an end of a stream that may be cut have moved there
 };
 
 // Position in the sequence of tiles: tile j of the stream (unit u, KV head h).  The lengths of units
@@ -348,18 +354,22 @@ __device__ __forceinline__ void process_block(uint32_t kt, uint32_t vt, int kb, 
 // The even deal of the tile sequence over the grid, found by all threads of the CTA from len[]: every
 // length is read once (and left in shared memory for units below NLEN), a block-wide prefix sum of tile
 // counts follows, then the two boundaries of this CTA's share.  Boundary c is tile T*c/n_cta; where it
-// falls inside a short stream (at most SNAP tiles, or SNAP_THIN) it moves to the nearer end of that stream, and where it falls
-// within EDGE tiles of an end of a longer one to that end.  Where all units have as many tiles, only as many CTAs
-// take part as share the streams out evenly (ctas_equal).  sc: [0..5] warp sums, [8] u0, [9] rem, [12] t0, [14] t1, [32..43] fewest and
-// most tiles of a unit, by warp.  The deal is a function of the tile counts of the lengths in slen and of nothing else (units from NLEN on
+// falls inside a stream that stays whole (Cuts) it moves to the nearer end of that stream, and where it falls
+// within `edge` tiles of an end of another one to that end.  Where all units have as many tiles, only as many CTAs
+// take part as share the streams out evenly (ctas_equal).  Where they differ, all of the grid does: the more CTAs, the more of
+// them are left to share the bandwidth of those that are through (16/4 heads x 128, 77 sequences of 0 to 1000 rows: 195 CTAs 22.4 us,
+// 259 19.2, 296 18.6; 8/4 x 64, 75 of 0 to 1150: 17.4 and 14.1) - except with heads of 128, and 1 or 2 of them, or 4 and more than 10
+// tiles per CTA, where the bandwidth is used up whatever the CTAs (16/4, 100 of 0 to 3000: 200 CTAs 54.8, 296 57.5; 8/8, 37 of 700 to
+// 800: 195 23.0, 296 24.0).  sc: [0..5] warp sums, [8] u0, [9] rem, [12] t0, [14] t1, [32..37] most tiles
+// of a unit, by warp.  The deal is a function of the tile counts of the lengths in slen and of nothing else (units from NLEN on
 // have no copy there and are dealt after the dependency wait): a length is read once, and what is compared with it later is that copy.
-template <bool PAGED>
+template <int DH, int GP, bool PAGED>
 __device__ __forceinline__ Share deal(const AttnParams &p, int *sc, int *slen, int cta) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     auto len_of = [&](int u) { return eff_len(p, u < NLEN ? slen[u] : ld_len<PAGED>(p, u)); };
     const int per = (p.n_units + THREADS - 1) / THREADS;
     const int ub = min(p.n_units, (int)threadIdx.x * per), ue = min(p.n_units, ub + per);
-    int mine = 0, fewest = INT_MAX, most = -1;                    // tiles of this thread's units; of one of them
+    int mine = 0, most = 0;                                       // tiles of this thread's units; of one of them, at most
     if (per <= LPT) {                                             // all loads in flight together
         int len[LPT];
         load_lengths<PAGED>(p, ub, ue, len, nullptr);
@@ -367,17 +377,16 @@ __device__ __forceinline__ Share deal(const AttnParams &p, int *sc, int *slen, i
         for (int i = 0; i < LPT; ++i)
             if (ub + i < ue) {
                 const int nt = tiles_of(eff_len(p, len[i]));
-                slen[ub + i] = len[i]; mine += nt; fewest = min(fewest, nt); most = max(most, nt);
+                slen[ub + i] = len[i]; mine += nt; most = max(most, nt);
             }
     } else {
         for (int u = ub; u < ue; ++u) {
             const int len = ld_len<PAGED>(p, u);
             if (u < NLEN) slen[u] = len;
             const int nt = tiles_of(eff_len(p, len));
-            mine += nt; fewest = min(fewest, nt); most = max(most, nt);
+            mine += nt; most = max(most, nt);
         }
     }
-    fewest = __reduce_min_sync(0xffffffffu, fewest);
     most = __reduce_max_sync(0xffffffffu, most);
     int incl = mine;
 #pragma unroll
@@ -385,25 +394,39 @@ __device__ __forceinline__ Share deal(const AttnParams &p, int *sc, int *slen, i
         const int v = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += v;
     }
-    int2 *extent = reinterpret_cast<int2 *>(sc + 32);
-    if (lane == 31) { sc[warp] = incl; extent[warp] = make_int2(fewest, most); }
+    if (lane == 31) { sc[warp] = incl; sc[32 + warp] = most; }
     __syncthreads();
     int before = 0, all = 0;
 #pragma unroll
     for (int w = 0; w < THREADS / 32; ++w) {
         if (w < warp) before += sc[w];
         all += sc[w];
-        fewest = min(fewest, extent[w].x); most = max(most, extent[w].y);
+        most = max(most, sc[32 + w]);
     }
-    const bool same = fewest == most;                             // as many tiles in every unit
+    const bool same = (long long)most * p.n_units == all;         // as many tiles in every unit
     Share sh;
     sh.T = (long long)all * p.Hkv;
     // every CTA that takes part owns at least one tile of the even deal, so the CTAs holding a cut stream
     // are consecutive
-    sh.n_cta = (int)min((long long)(same ? min(p.ctas_equal, (int)gridDim.x) : gridDim.x), sh.T);
-    const bool thin = sh.T < (long long)THIN * sh.n_cta;
-    const int snap = thin ? SNAP_THIN : SNAP;
-    sh.edge = thin ? EDGE_THIN : EDGE;
+    using C = Cuts<DH, GP>;
+    int n_cta = gridDim.x;
+    const bool thick = DH == 128 && (!C::DEAR || (!C::VERY_DEAR && sh.T >= (long long)C::THICK * n_cta));
+    if (same) n_cta = min(p.ctas_equal, n_cta);
+    else if (thick) n_cta = min(p.ctas_differ, n_cta);
+    sh.n_cta = (int)min((long long)n_cta, sh.T);
+    // streams of at most `keep` tiles stay whole, and those of `from` to `to` tiles
+    int keep = C::DEAR && same ? p.whole_equal : C::WHOLE, from = 1, to = 0;
+    sh.edge = 0;
+    if (C::DEAR && !same && !thick) {
+        const float even = (float)sh.T / (float)sh.n_cta;
+        if (even >= C::THIN) {
+            sh.edge = C::EDGE;
+            if (C::VERY_DEAR) keep = max(keep, min(C::WHOLE_DEAR, (int)(even * 0.625f)));
+            from = (int)(even * (C::VERY_DEAR ? 1.54f : 1.25f)) + 1;
+            to = C::VERY_DEAR ? C::WHOLE_DEAR : min(C::WHOLE_DEAR, (int)even + 7);
+        }
+    }
+    auto whole = [&](int nt) { return nt <= keep || (C::DEAR && nt >= from && nt <= to); };
     {
         const long long lo = (long long)(before + incl - mine) * p.Hkv, hi = lo + (long long)mine * p.Hkv;
 #pragma unroll
@@ -422,8 +445,8 @@ __device__ __forceinline__ Share deal(const AttnParams &p, int *sc, int *slen, i
                     int rem = (int)(x - pre), uu = u;
                     const int j = rem % nt;
                     long long bx = x;
-                    if (j != 0 && (nt <= snap ? 2 * j <= nt : j <= sh.edge)) { bx = x - j; rem -= j; }
-                    else if (j != 0 && (nt <= snap || nt - j <= sh.edge)) { bx = x + (nt - j); rem += nt - j; }
+                    if (j != 0 && (whole(nt) ? 2 * j <= nt : j <= sh.edge)) { bx = x - j; rem -= j; }
+                    else if (j != 0 && (whole(nt) || nt - j <= sh.edge)) { bx = x + (nt - j); rem += nt - j; }
                     if (rem == nt * p.Hkv) {                      // moved to the start of the next unit that has keys
                         rem = 0;
                         do { ++uu; } while (uu < p.n_units && len_of(uu) == 0);
@@ -510,7 +533,7 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
     Walker<PAGED> w;
     bool started = false;
     if (ahead) {
-        sh = deal<PAGED>(p, sc, slen, cta);
+        sh = deal<DH, GP, PAGED>(p, sc, slen, cta);
         if (sh.t0 < sh.t1) started = w.start(p, sh, slen);
     }
 
@@ -604,7 +627,7 @@ coarse_attn_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k,
             }
         }
         if (threadIdx.x == 0) { sc[8] = -1; sc[9] = 0; sc[12] = 0; sc[14] = -1; }
-        sh = deal<PAGED>(p, sc, slen, cta);
+        sh = deal<DH, GP, PAGED>(p, sc, slen, cta);
         started = sh.t0 < sh.t1 && w.start(p, sh, slen);
     } else if (started && w.valid(p)) {
         w.load(p);                          // same tile counts, but the unit may have grown within its last tile
@@ -972,10 +995,21 @@ cudaError_t run(photon_ctx *ctx, AttnParams p, cudaStream_t st, long long *launc
     const long long t_max = (long long)p.n_units * p.Hkv * ((max_len + BN - 1) / BN);
     const long long streams = (long long)p.n_units * p.Hkv;
     p.ctas_equal = ctx->attn_ctas > 0 ? ctx->attn_ctas : coarse_attn_grid(ctx->max_ctas, streams);
+    if constexpr (Cuts<DH, GP>::DEAR) {
+        // of `rounds` streams to a CTA, and `even` to one on average: how long they may be for the difference to be 5 tiles
+        using C = Cuts<DH, GP>;
+        const int n = std::max(1, p.ctas_equal);
+        const float even = (float)streams / n, rounds = (float)((streams + n - 1) / n);
+        p.whole_equal = C::VERY_DEAR ? (even >= 0.5f ? C::WHOLE_DEAR : C::WHOLE)
+                                     : std::max(C::WHOLE, (int)std::min((float)C::WHOLE_DEAR, 5.f / std::max(0.01f, rounds - even)));
+    }
+    p.ctas_differ = ctx->attn_ctas > 0 ? ctx->attn_ctas : coarse_attn_grid(ctx->max_ctas, streams, false);
     // More streams than that: which CTAs take part is decided on the device, by whether the lengths are equal.  (Not with very many
     // streams: they even out by themselves, and the CTAs that leave at once cost a step of 512 x 8 streams 2.7 of 241 us.)
     const bool by_lengths = ctx->attn_ctas <= 0 && streams > p.ctas_equal && streams <= 8ll * ctx->max_ctas;
-    const long long cap = by_lengths ? ctx->max_ctas : p.ctas_equal;
+    // (with up to 4 heads of 128 the whole grid is for calls of few tiles per CTA only, see deal)
+    const bool all = DH == 64 || GP >= 8 || (GP == 4 && streams <= 3ll * ctx->max_ctas);
+    const long long cap = !by_lengths ? p.ctas_equal : all ? ctx->max_ctas : std::max(p.ctas_equal, p.ctas_differ);
     const int grid = (int)std::max<long long>(1, std::min<long long>(t_max, cap));
     const cudaError_t e = launch_dependent(coarse_attn_kernel<DH, GP, PAGED>, dim3(grid), dim3(THREADS), smem, st, 0, p, mk, mv, mk_end, mv_end);
     ++*launches;
@@ -992,17 +1026,15 @@ int coarse_attn_fold_limit() { return NLEN; }
 // through its set-up, while this one still runs (measured on caches of 64 to 256 MiB: 7/8 of the slots is 1 to 4 %
 // faster than all of them).  Up to that many (unit, KV head) streams the grid is a multiple of their number, so that every
 // stream falls to the same whole number of CTAs and the cuts of the deal line up with the streams' ends; with more it is what
-// makes as few rounds of whole streams as there can be, the last eighth of the slots included where that saves more than its
-// share (200 sequences of 150 rows, 4 KV heads: 16.4 -> 15.3 us with 267 CTAs
-// instead of 200; 130 of 1000: 48.9 -> 45.4).  Where lengths differ all slots are taken then: the more CTAs, the more of them are left
-// to share the bandwidth of those that are through (77 sequences of 0 to 1000 rows: 195 CTAs 22.4 us, 259 19.2, 296 18.6).
-int coarse_attn_grid(int resident_ctas, long long n_streams) {
+// makes as few rounds of whole streams as there can be, the last eighth of the slots included (last_eighth) where that saves more than
+// its share (200 sequences of 150 rows, 4 KV heads: 16.4 -> 15.3 us with 267 CTAs instead of 200; 130 of 1000: 48.9 -> 45.4).
+int coarse_attn_grid(int resident_ctas, long long n_streams, bool last_eighth) {
     const int top = std::max(1, resident_ctas * 7 / 8);
     if (n_streams <= 0) return 1;
     if (n_streams <= top) return (int)(n_streams * (top / n_streams));
     // more streams than CTAs: as few whole streams per CTA as there can be, and no more CTAs than that takes
     const long long rounds = (n_streams + top - 1) / top, fewest = (n_streams + resident_ctas - 1) / resident_ctas;
-    const long long r = fewest * 8 < rounds * 7 ? fewest : rounds;
+    const long long r = last_eighth && fewest * 8 < rounds * 7 ? fewest : rounds;
     return (int)std::max<long long>(top - top / 4, (n_streams + r - 1) / r);
 }
 

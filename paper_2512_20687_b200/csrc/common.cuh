@@ -74,6 +74,8 @@ struct AttnParams {
     int page_rows, pages_per_unit, n_pages;
     int n_q, Hq, Hkv, dh;
     int ctas_equal;          // filled by the launcher: CTAs of the coarse attention that take part when every unit has as many tiles
+    int whole_equal;         // filled by the launcher: streams of at most so many tiles are not cut then
+    int ctas_differ;         // filled by the launcher: and when not, where the whole grid is too many
     int splits_sh;           // key ranges of a shared prefix = cluster size of its kernel (0: no shared prefix)
     int upc;                 // filled by the launcher: units per CTA on shared keys
     int own_rows;            // filled by the launcher: the units' own keys (at most this many rows each) are read by the
@@ -197,7 +199,7 @@ cudaError_t launch_shared_prefix_attention(photon_ctx *ctx, const AttnParams &p,
                                            long long *launches);
 int coarse_attn_ctas_per_sm();
 int coarse_attn_fold_limit();     // largest batch for which the step's append can be folded into the attention
-int coarse_attn_grid(int resident_ctas, long long n_streams);
+int coarse_attn_grid(int resident_ctas, long long n_streams, bool last_eighth = true);
 int shared_prefix_units_per_cta(int G);
 int shared_prefix_own_rows();
 // Whether an attention call on this cache is one launch: a shared prefix, and own caches short enough (by the caller's

@@ -252,3 +252,40 @@ def test_deal_of_more_streams_than_ctas_behind_an_append(n, lengths, paged):
     want, size = (torch.einsum("nhgs,nhsd->nhgd", w, x).reshape(n, Hq, dh) for x in (want_v, want_v.abs()))
     assert ((out.double() - want).abs() <= 2.0 ** -8 * (want.abs() + size) + 1e-5).all()
     assert (lse.double() - torch.logsumexp(logit, -1).view(n, Hq)).abs().max() < 2e-3
+
+
+# (16, 4): kept whole, cut in halves, cut in four; ragged with all CTAs, few tiles per CTA, many; nearly equal.  (16, 1): cut in two and four,
+# ragged, nearly equal.  (8, 8): never whole above 8 tiles
+DEALS = [(16, 4, 32, 640, "equal"), (16, 4, 32, 1024, "equal"), (16, 4, 24, 1024, "equal"), (16, 4, 16, 1024, "equal"), (16, 4, 75, 576, "equal"),
+         (16, 4, 75, 1000, "ragged"), (16, 4, 250, 300, "ragged"), (16, 4, 60, 3000, "ragged"), (16, 4, 32, 1000, "ragged"), (16, 4, 75, 800, "near"),
+         (16, 1, 100, 1024, "equal"), (16, 1, 64, 1024, "equal"), (16, 1, 300, 1000, "ragged"), (16, 1, 130, 900, "near"), (8, 8, 37, 1024, "equal"),
+         (8, 8, 37, 1000, "ragged")]
+
+
+@pytest.mark.parametrize("Hq,Hkv,n,S,lengths", DEALS)
+def test_streams_that_stay_whole_and_streams_that_are_cut(Hq, Hkv, n, S, lengths):
+    """Heads of 128 features, where what a cut costs decides.  Twice (the tickets are as they should be), and within the two
+    roundings to bf16 of torch in 64 bits: the output's (2^-8 of the value) and the weights' (2^-8 of the weighted sum of the absolute values)."""
+    dh = 128
+    cfg = wl.scaled(wl.CONFIGS[1], B=n, Hq=Hq, Hkv=Hkv, dh=dh, D=Hq * dh)
+    rng = np.random.default_rng(n + S)
+    lens = dev_i32(np.full(n, S) if lengths == "equal" else rng.integers(0 if lengths == "ragged" else S * 7 // 8, S + 1, n))
+    g = torch.Generator("cuda").manual_seed(n)
+    k, v, q = ((torch.randn(*s, generator=g, device="cuda")).to(torch.bfloat16) for s in ((n, Hkv, S, dh), (n, Hkv, S, dh), (n, Hq, dh)))
+    outs = [(torch.empty_like(q), torch.empty(n, Hq, device="cuda")) for _ in range(2)]
+    with Ctx(cfg) as c:
+        for out, lse in outs:
+            ph.photon_coarse_attn(c.h, ph.make_kv(k, v, lens), q, out, lse, dh ** -0.5)
+            assert c.status() == 0
+    assert torch.equal(outs[0][0].view(torch.int16), outs[1][0].view(torch.int16)) and torch.equal(outs[0][1], outs[1][1])
+    out, lse = outs[0]
+    for u in range(n):                                                    # (a unit at a time: 64-bit copies of the caches are large)
+        L = int(lens[u])
+        if L == 0:
+            assert bool((out[u] == 0).all()) and bool(torch.isneginf(lse[u]).all())
+            continue
+        logit = torch.einsum("hgd,hsd->hgs", q[u].double().view(Hkv, Hq // Hkv, dh), k[u, :, :L].double()) * dh ** -0.5
+        w = torch.softmax(logit, -1)
+        want, size = (torch.einsum("hgs,hsd->hgd", w, x).reshape(Hq, dh) for x in (v[u, :, :L].double(), v[u, :, :L].double().abs()))
+        assert ((out[u].double() - want).abs() <= 2.0 ** -8 * (want.abs() + size) + 1e-5).all(), u
+        assert (lse[u].double() - torch.logsumexp(logit, -1).view(Hq)).abs().max() < 2e-3
