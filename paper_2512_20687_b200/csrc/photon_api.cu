@@ -741,8 +741,11 @@ photon_status step_impl(photon_ctx *ctx, const photon_step_args *a, photon_strea
     if (beside) {
         if (cudaStreamWaitEvent(st, ctx->ev_join, 0) != cudaSuccess && s == PHOTON_OK) s = PHOTON_ERR_CUDA;
     } else if (s == PHOTON_OK && a->Nc > 0) {
+        // (It reads keys and values by the path for data that no kernel writes meanwhile: it may start ahead of its turn only behind a
+        // coarse attention, which lets what follows it start when all that was enqueued before the call is written.  The converter
+        // alone lets it start before that.)
         s = attention_common(ctx, a->chunks, q_chunk, slot, a->Nc, out_chunk, nullptr, a->scale_chunk, true, st, nullptr, nullptr,
-                             direct, tiny);
+                             direct, tiny && a->coarse->n_units > 0);
     }
     if (copying && cudaStreamWaitEvent(st, ctx->ev_copy, 0) != cudaSuccess && s == PHOTON_OK) s = PHOTON_ERR_CUDA;
     if (s == PHOTON_OK && hp && !copy_out(hp, copying ? early_end : 0, apart || direct ? hp->out_split : hp->out_bytes, st))

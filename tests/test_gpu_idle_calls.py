@@ -93,3 +93,45 @@ def test_decode_steps_one_at_a_time(idx):
             for got, want in zip((out, U, oc), first):
                 assert torch.equal(bits(got), bits(want)), f"decode step, call {it}"
         assert np.array_equal(d["len"].cpu().numpy(), len0.cpu().numpy() + 1)
+
+
+@pytest.mark.parametrize("B", [0, 3])
+def test_small_steps_without_a_coarse_sequence_behind_writers_of_their_chunks(B):
+    """No coarse sequence is there, so no kernel of the step waits before the chunk attention but the converter (B latents), which
+    lets the next kernel start at once; the queries, the chunks' new rows and their lengths come from kernels of the library
+    enqueued just before.  Against the same calls with a wait between them."""
+    Hq, Hkv, dh, P, C, Nc = 4, 2, 64, 4, 8, 24
+    D = Hq * dh
+    cfg = wl.scaled(wl.CONFIGS[0], B=1, Hq=Hq, Hkv=Hkv, dh=dh, D=D, P=P, C=C)
+    gen = torch.Generator("cuda").manual_seed(3)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda").to(torch.bfloat16)
+    k0, v0, xs, wq = rand(Nc, Hkv, P + C, dh), rand(Nc, Hkv, P + C, dh), rand(C, Nc, D), rand(D, D)
+    k_new, v_new = rand(C, Nc, Hkv, dh), rand(C, Nc, Hkv, dh)
+    x, w, one = rand(max(B, 1), D), rand(D, P * D), torch.zeros(1, 1, 1, dh, dtype=torch.bfloat16, device="cuda")
+    held = torch.empty(16 << 20, dtype=torch.uint8, device="cuda").random_()
+    with Ctx(cfg, max_queries=Nc) as c:
+        first = None
+        for turn in range(20):
+            kc, vc, ln = k0.clone(), v0.clone(), torch.full((Nc,), P, dtype=torch.int32, device="cuda")
+            ckv, none = ph.make_kv(kc, vc, ln), ph.make_kv(one, one.clone(), torch.zeros(1, dtype=torch.int32, device="cuda"))
+            none.n_units = 0
+            q, outs, U = torch.empty(Nc, D, dtype=torch.bfloat16, device="cuda"), [], torch.empty(max(B, 1), P, D, dtype=torch.bfloat16, device="cuda")
+            torch.cuda.synchronize()
+            if turn:
+                ph.photon_read_probe(c.h, held[:turn * 839680])
+            for t in range(C):
+                outs.append(torch.empty(Nc, Hq, dh, dtype=torch.bfloat16, device="cuda"))
+                args = ph.make_step_args(none, one, one, one, one, 1.0, w, ph.PHOTON_W_IN_MAJOR, U, B, chunks=ckv, q_chunk=q.view(Nc, Hq, dh),
+                                         out_chunk=outs[-1], Nc=Nc, scale_chunk=dh ** -0.5, x=x)
+                ph.photon_linear(c.h, xs[t], wq, ph.PHOTON_W_IN_MAJOR, None, q)
+                ph.photon_kv_append(c.h, ckv, k_new[t], v_new[t])
+                if not turn:
+                    torch.cuda.synchronize()
+                ph.photon_decode_step(c.h, args)
+                if not turn:
+                    torch.cuda.synchronize()
+            assert c.status() == 0
+            got = [bits(o).clone() for o in outs] + [bits(U).clone() if B else None]
+            first = first or got
+            for a, b in zip(got, first):
+                assert a is None or torch.equal(a, b), turn
