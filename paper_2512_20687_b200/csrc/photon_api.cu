@@ -620,14 +620,21 @@ photon_status step_impl(photon_ctx *ctx, const photon_step_args *a, photon_strea
     // low-priority stream that forks from `stream` here and joins it again before the call returns, so
     // for the caller the whole step is still ordered on `stream`.  Large chunk workloads stay in line:
     // two kernels that are both bound by HBM gain nothing from running side by side.  So do steps of at most 8 MB that are launched
-    // one by one: the device is through with all three kernels before the host has enqueued them (9 of 20 us), and the fork and the
-    // join are four calls more (2 sequences of the 256-wide model, 8 chunks each, 20.3 -> 18.7 us; replayed they would cost 1.5).
+    // one by one, with at most 256 rows to a sequence (its shared prefix included) and 2048 query heads of chunks: the device is through
+    // with all three kernels before the host has enqueued them (18.5 us), and the fork and the join are four calls more.  us, beside / in
+    // line: 4/2 heads x 64, 2 sequences of 16 rows with 8 chunks each 20.3 / 18.7, 64 of 200 with 2 20.0 / 18.6; 4/2 x 128, 16 of 64 with 32
+    // 18.5 / 17.3; 8/1 x 64, 16 of 200 with 8 18.4 / 18.6.  Longer streams or more chunks take longer than the host: 8/1 x 64, 4 of 500 18.7 /
+    // 20.6, 1 of 1000 18.7 / 21.7, 200 of 16 with 8 chunks 18.5 / 21.8; 4/2 x 64, 2 of 4000 25.0 / 27.3.  (Replayed it would cost 1.5 us.)
+    const photon_kv &co = *a->coarse;
+    const size_t own_rows = co.max_len ? co.max_len : co.cap;
+    const size_t prefix_rows = !co.k_shared ? 0 : co.max_shared_len ? co.max_shared_len : co.cap_shared;
     const size_t chunk_bytes = a->Nc > 0 ? (size_t)a->Nc * c.Hkv * a->chunks->cap * c.dh * 4 : 0;
     const size_t step_bytes = chunk_bytes + (size_t)c.D * c.P * c.D * 2 +
-                              (size_t)a->coarse->n_units * c.Hkv * (a->coarse->max_len ? a->coarse->max_len : a->coarse->cap) * c.dh * 4;
+                              (co.n_units * own_rows + (prefix_rows ? co.n_shared : 0) * prefix_rows) * c.Hkv * c.dh * 4;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) return PHOTON_ERR_CUDA;
-    const bool tiny = !hp && capture == cudaStreamCaptureStatusNone && step_bytes <= (size_t(8) << 20);
+    const bool tiny = !hp && capture == cudaStreamCaptureStatusNone && step_bytes <= (size_t(8) << 20) && own_rows + prefix_rows <= 256 &&
+                      (size_t)a->Nc * c.Hq <= 2048;
     const bool beside = a->Nc > 0 && chunk_bytes <= (size_t(32) << 20) && !tiny;
     photon_status s = PHOTON_OK;
     // With host buffers and a declared split the two halves of either buffer travel apart.  Where both host buffers are
