@@ -384,9 +384,12 @@ cudaError_t run_large(photon_ctx *ctx, const ConvParams &p, cudaStream_t st, lon
 
 // Where the pair kernel is the faster one, by both kernels' estimates; the pairs' is a little low.  us, projection kernel / pairs:
 // 700 x 2048 -> 3072 11.7 / 12.8, 900 x 2048 -> 3072 16.3 / 14.0, 1204 x 2048 -> 2048 + residual 20.5 / 14.7, 1204 x 1024 -> 1024 8.2 / 8.3,
-// 3072 x 1024 -> 1024 15.6 / 11.0, 300 x 2048 -> 11264 18.9 / 22.7, 4096 x 256 -> 512 5.1 / 6.2.
+// 3072 x 1024 -> 1024 15.6 / 11.0, 300 x 2048 -> 11264 18.9 / 22.7, 4096 x 256 -> 512 5.1 / 6.2.  From more than two waves of its largest tiles
+// on the projection kernel's estimate is too low, and the pairs are faster wherever it took that kernel (1600 x 2048 -> 8192 49.4 / 44.8,
+// out-major 54.3 / 46.8; 3334 x 4096 -> 4096 + residual 99.5 / 87.8, out-major 111.5 / 92.3).
 bool linear_wants_pairs(const int *fit, const ConvParams &p, bool gated) {
     if (fit[2] < 1 || p.B <= BM) return false;
+    if ((long long)((p.B + 127) / 128) * ((p.N + 255) / 256) > 2ll * fit[1]) return true;
     const float slab = linear_slab_us(fit, p, gated);
     return slab < 0.f || 1.04f * pair_plan(fit[2], p.B, p.D, p.N, !p.w_out_major, grain_of(p)).us < slab;
 }

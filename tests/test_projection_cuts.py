@@ -92,3 +92,9 @@ def test_pairs_are_taken_for_many_rows_only_and_where_the_device_holds_them():
     for K, N in ((2048, 3072), (2048, 2048), (1024, 3072), (5632, 2048), (2048, 11264)):
         assert pair_cut(16384, K, N, True)[0] and not pair_cut(128, K, N, True)[0]
         assert not pair_cut(16384, K, N, True, clusters=(0, 148, 0, 0, 0, 0, 0, 0, 0))[0]
+
+
+@pytest.mark.parametrize("B,K,N,residual", [(1600, 2048, 8192, False), (1540, 2048, 8192, False), (3334, 4096, 4096, True), (4737, 64, 2048, False)])
+def test_pairs_are_taken_from_more_than_two_waves_on(B, K, N, residual):
+    for out_major in (False, True):
+        assert pair_cut(B, K, N, out_major, residual)[0]
