@@ -487,10 +487,12 @@ cudaError_t launch(photon_ctx *ctx, AttnParams p, cudaStream_t st, long long *la
     //  - with fewer heads at a time, or longer buffers: there the compiler gives the small CTA too few registers and its row loads
     //    wait for one another (8/8 x 128, 24 rows: 128 chunks 4.2 / 9.0; 16/4 x 128, 48 rows: 1000 chunks 37 / 57);
     //  - of 24 rows, up to one wave of eight-warp CTAs (16/4 x 128: 256 chunks 5.8 / 7.7; beyond it about equal);
+    //  - where they start together with the coarse part of a captured step, up to one wave: spread over all SMs the small CTAs are in the
+    //    way of the coarse attention's second CTA per SM (64 sequences with 2 chunks each, 28.1 / 29.6);
     //  - where queries and results cross the bus: hundreds of resident CTAs that wait for it (280 sequences with 8 chunks each,
     //    host-driven: 330 / 350; 64 with 2: 57.4 / 63.0).
     if constexpr (GT == 4 && RP <= 24) {
-        if (!p.over_bus && !(one_wave && RP == 24)) {
+        if (!p.over_bus && !(one_wave && (p.replayed_first || RP == 24))) {
             const cudaError_t e = start(chunk_attn_kernel<DH, RP, GT, 1>, (unsigned)items, 32);
             ++*launches;
             return e != cudaSuccess ? e : cudaGetLastError();

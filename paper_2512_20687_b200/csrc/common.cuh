@@ -82,6 +82,7 @@ struct AttnParams {
                              // shared-prefix kernel, which then writes the final result; 0: a second kernel reads them
     bool over_bus;           // chunk attention: queries and results in host memory
     bool dependent;          // chunk attention: behind another kernel of the same call
+    bool replayed_first;     // chunk attention: in a captured step, starting with its coarse attention
     float scale_log2;        // scale * log2(e): logits are kept in the base-2 domain
     float *partials;
     float *cta_partials;

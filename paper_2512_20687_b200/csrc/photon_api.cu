@@ -40,7 +40,8 @@ int ceil_div(int a, int b) { return (a + b - 1) / b; }
 photon_status attention_common(photon_ctx *ctx, const photon_kv *cache, const photon_bf16 *q,
                                const int32_t *slot, int n_q, photon_bf16 *out, float *lse,
                                float scale, bool chunk, cudaStream_t st, const photon_bf16 *k_new = nullptr,
-                               const photon_bf16 *v_new = nullptr, bool over_bus = false, bool dependent = false) {
+                               const photon_bf16 *v_new = nullptr, bool over_bus = false, bool dependent = false,
+                               bool replayed_first = false) {
     if (!ctx) return PHOTON_ERR_INVALID_ARG;
     if (!kv_ok(ctx, cache, !chunk) || (chunk && cache->page_table)) return PHOTON_ERR_INVALID_ARG;
     if (n_q < 0 || (n_q > 0 && (!q || !out))) return PHOTON_ERR_INVALID_ARG;
@@ -84,6 +85,7 @@ photon_status attention_common(photon_ctx *ctx, const photon_kv *cache, const ph
     }
     p.over_bus = over_bus;
     p.dependent = dependent;
+    p.replayed_first = replayed_first;
     p.max_len = cache->max_len ? cache->max_len : cache->cap;
     p.splits_sh = 0;
     if (!chunk) {
@@ -696,21 +698,32 @@ photon_status step_impl(photon_ctx *ctx, const photon_step_args *a, photon_strea
             return PHOTON_ERR_CUDA;
         if (apart && !direct && !copy_in(hp, hp->in_split, hp->in_bytes, ctx->side)) s = PHOTON_ERR_CUDA;
     }
+    // Called one by one the chunk attention goes to its stream first: it is launched while the coarse part's kernel is still on its
+    // way.  In a captured step both start at the same time, and where the chunk attention is the first node its CTAs take
+    // registers from the coarse attention's first wave.  It follows there
+    //  - with buffers of up to 8 rows, whose CTAs are small and through soon, and a coarse part that takes longer (16/4 heads x 128, replayed,
+    //    first / behind, 64 sequences 30.6 / 27.7 us, 16 long ones 60.7 / 58.2; 16/1, 64 of 64 rows 18.7 / 20.1);
+    //  - with up to 24 rows and two heads at a time (8/4 x 128, 64 of 256 20.3 / 19.6), or one of 128 features beside few streams or many
+    //    bytes (8/8 x 128, 16 of 512 with 8 chunks 22.9 / 20.3, 64 of 1024 57.4 / 54.8).
+    // Others hold up the converter when they follow (8/8 x 128, 24 rows, 24 of 64 14.6 / 17.0, 48 rows 17.7 / 22.8; 16/4 x 128, 24 rows, 64
+    // of 256 33.8 / 40.7).  (Called one by one that order is no faster, the long ones 59.8 and 60.5.)
+    const int G = c.Hq / c.Hkv;
+    const size_t rows = own_rows + prefix_rows, cap = a->Nc > 0 ? a->chunks->cap : 0;
+    const size_t coarse_bytes = co.n_units * own_rows * c.Hkv * c.dh * 4;
+    const bool behind = beside && capture != cudaStreamCaptureStatusNone &&
+                        (cap <= 8 ? rows >= 16 * (size_t)G
+                                  : cap <= 24 && rows >= 128 && (G % 4 == 2 || (G == 1 && c.dh == 128 && ((size_t)co.n_units * c.Hkv <= 128 || coarse_bytes >= 200000000))));
+    const bool chunks_first = !behind;
     // every way out from here on joins the side stream again, failed calls included
     auto chunks_beside = [&]() {
         if (s == PHOTON_OK)
             s = attention_common(ctx, a->chunks, q_chunk, slot, a->Nc, out_chunk, nullptr, a->scale_chunk, true, ctx->side, nullptr,
-                                 nullptr, direct);
+                                 nullptr, direct, false, chunks_first && capture != cudaStreamCaptureStatusNone);
         if (s == PHOTON_OK && apart && !direct && !copy_out(hp, hp->out_split, hp->out_bytes, ctx->side)) s = PHOTON_ERR_CUDA;
         if (cudaEventRecord(ctx->ev_join, ctx->side) != cudaSuccess && s == PHOTON_OK) s = PHOTON_ERR_CUDA;
         if (s != PHOTON_OK) cudaStreamWaitEvent(st, ctx->ev_join, 0);
         return s;
     };
-    // Called one by one the chunk attention goes to its stream first: it is launched while the coarse part's kernel is still on its
-    // way.  In a captured step both start at the same time, and where the chunk attention is the first node its CTAs take
-    // registers from the coarse attention's first wave: there it follows (replayed, 64 sequences 25.2 -> 23.6 us, 16 long ones
-    // 60.1 -> 57.9, 77 ragged paged ones 40.3 -> 37.0; called one by one that order is no faster, the long ones 59.8 and 60.5).
-    const bool chunks_first = capture == cudaStreamCaptureStatusNone;
     if (beside && (chunks_first || s != PHOTON_OK) && chunks_beside() != PHOTON_OK) return s;
     // The append is one row per unit, in place: for a batch whose lengths fit the attention kernel's shared memory it
     // is folded into that kernel (the warp that reaches a unit's last tile installs the

@@ -135,3 +135,40 @@ def test_small_steps_without_a_coarse_sequence_behind_writers_of_their_chunks(B)
             first = first or got
             for a, b in zip(got, first):
                 assert a is None or torch.equal(a, b), turn
+
+
+@pytest.mark.parametrize("Hq,Hkv,dh,P,C,B,S,per", [(16, 4, 128, 4, 4, 20, 300, 2), (16, 4, 128, 8, 16, 20, 300, 2), (16, 4, 128, 4, 12, 9, 100, 3), (8, 8, 128, 8, 16, 12, 200, 2),
+                                                   (8, 8, 128, 8, 16, 40, 200, 2), (8, 4, 128, 8, 16, 20, 200, 2), (8, 4, 128, 8, 16, 20, 40, 2),
+                                                   (4, 2, 64, 4, 4, 5, 20, 4)])
+def test_captured_steps_in_either_order_of_their_attentions(Hq, Hkv, dh, P, C, B, S, per):
+    """A captured step enqueues the chunk attention in front of the coarse attention or behind it; replayed, the bits of the same step
+    called by itself."""
+    cfg = wl.scaled(wl.CONFIGS[1], B=B, Hq=Hq, Hkv=Hkv, dh=dh, D=Hq * dh, P=P, C=C)
+    D, Nc = Hq * dh, B * per
+    gen = torch.Generator("cuda").manual_seed(B + S)
+    rand = lambda *s, std=1.0: (torch.randn(*s, generator=gen, device="cuda") * std).to(torch.bfloat16)
+    k, v, q, k_new, v_new = rand(B, Hkv, S, dh), rand(B, Hkv, S, dh), rand(B, Hq, dh), rand(B, Hkv, dh), rand(B, Hkv, dh)
+    kc, vc, qc, w = rand(Nc, Hkv, P + C, dh), rand(Nc, Hkv, P + C, dh), rand(Nc, Hq, dh), rand(D, P * D, std=D ** -0.5)
+    len0 = torch.randint(0, S, (B,), generator=gen, device="cuda", dtype=torch.int32)
+    ln, lc = len0.clone(), torch.randint(P, P + C + 1, (Nc,), generator=gen, device="cuda", dtype=torch.int32)
+    out, oc, U = torch.empty_like(q), torch.empty_like(qc), torch.empty(B, P, D, dtype=torch.bfloat16, device="cuda")
+    with Ctx(cfg, max_queries=Nc) as c:
+        args = ph.make_step_args(ph.make_kv(k, v, ln), k_new, v_new, q, out, dh ** -0.5, w, ph.PHOTON_W_IN_MAJOR, U, B, chunks=ph.make_kv(kc, vc, lc),
+                                 q_chunk=qc, out_chunk=oc, Nc=Nc, scale_chunk=dh ** -0.5)
+        ph.photon_decode_step(c.h, args)
+        want = [bits(t).clone() for t in (out, U, oc)]
+        stream = torch.cuda.Stream()
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph, stream=stream):
+            ln.copy_(len0)
+            ph.photon_decode_step(c.h, args, stream=stream)
+        for _ in range(5):
+            for t in (out, U, oc):
+                t.fill_(7.0)
+            graph.replay()
+            torch.cuda.synchronize()
+            assert c.status() == 0 and torch.equal(ln, len0 + 1)
+            for got, b in zip((out, U, oc), want):
+                assert torch.equal(bits(got), b)
+        del graph
