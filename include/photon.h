@@ -423,8 +423,8 @@ photon_status photon_coarse_attn_noalloc(const photon_config *cfg, const photon_
 
 /* Sets the persistent grid of photon_coarse_attn / photon_flat_attn to n CTAs
  * (0 or more than the device holds, two per SM: back to the default, where
- * the library picks a grid of at most 7/8 of what the device holds, lined up
- * with the number of (unit, KV head) streams of the call).  The keys of a call
+ * the library picks a grid by the number of (unit, KV head) streams of the
+ * call and by whether their lengths are equal, up to what the device holds).  The keys of a call
  * are dealt out evenly over the grid, so n also moves the points where a long
  * cache is cut and merged by log-sum-exp; a smaller grid leaves SMs free for
  * work on another stream.  Takes effect from the next call. */

@@ -26,7 +26,8 @@
 // kernel).  No bias, no residual.
 //
 // ROTARY: a fused q/k/v projection that leaves rotated, split and appended (see RopeOut).  A tile is one head; a group of columns is 8
-// features and their rotation partners.  The angles are computed where they are used, from the row's position.
+// features and their rotation partners.  Cosines and sines of the first positions (31 of heads of 128, 62 of 64) come from a table that
+// four warps fill under the contraction; those of later positions are computed where they are used.
 #include <algorithm>
 #include <type_traits>
 

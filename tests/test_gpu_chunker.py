@@ -250,7 +250,7 @@ def test_large_tile_kernel_adds_bias_and_residual_and_is_deterministic(oracle):
         ph.photon_linear(c.h, dx, dw, ph.PHOTON_W_IN_MAJOR, db, y2, residual=y2)
         assert c.status() == 0
     assert np.array_equal(host_bits(y1), host_bits(y2))
-    assert_close(host_f64(y1)[pick], want, "large tiles, bias + residual")
+    assert_close(host_f64(y1)[pick], want, "CTA pairs, bias + residual")
 
 
 def test_linear_one_hot_rows_return_weight_rows_bit_exactly():

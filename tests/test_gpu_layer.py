@@ -283,7 +283,7 @@ def test_converter_output_reaches_the_chunk_buffers(oracle, idx, B, chunks_per_s
 
 @pytest.mark.parametrize("layout", ["in", "out"])
 def test_decoder_step_with_thousands_of_chunks_fuses_the_activation(oracle, layout):
-    """5120 in-flight chunks: the gate/up projection takes the persistent large-tile kernel with
+    """5120 in-flight chunks: the gate/up projection takes the persistent kernel of CTA pairs with
     the activation in its epilogue (the [rows, 2F] intermediate is never written); both weight orders."""
     cfg = cfg_small(0, B=640, chunks_per_seq=8)                          # D 256, 4q/2kv x 64, P = C = 4
     Nc, F = cfg.Nc, 1024
@@ -608,3 +608,36 @@ def test_decoder_step_with_scratch_arrays_over_the_normalised_rows(name, Hq, Hkv
             assert c.status() == 0 and torch.equal(ln, len0 + 1)
             got.append([y, k, v])
     assert_same_but_for_roundings(*got)
+
+
+# positions up to the last of the tables of cosines and sines (31 positions of heads of 128, 62 of 64, few rows; 64, many) and beyond
+@pytest.mark.parametrize("Hq,Hkv,dh,P", [(8, 8, 128, 31), (8, 8, 128, 32), (8, 8, 128, 48), (4, 2, 64, 62), (4, 2, 64, 63), (8, 4, 128, 63)])
+@pytest.mark.parametrize("n", [3, 160])
+def test_prefill_of_long_prefixes_rotates_by_every_position(Hq, Hkv, dh, P, n):
+    """Against the split, the append and the attention called one after the other on the projection the call has left in its
+    scratch: same bits, lengths and status.  One buffer has no room."""
+    cap, T, scale = min(64, P + 3), n * P, dh ** -0.5
+    cfg = wl.scaled(wl.CONFIGS[4], B=1, Hq=Hq, Hkv=Hkv, dh=dh, D=Hq * dh, P=P, C=64 - P)
+    g = torch.Generator("cuda").manual_seed(n + P)
+    rand = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    layer = layer_of(g, Hq, Hkv, dh, 128, n == 3)
+    ids = torch.randperm(n, generator=g, device="cuda").to(torch.int32)
+    len0 = torch.zeros(n, dtype=torch.int32, device="cuda")
+    len0[ids[0].long()] = cap - P + 1
+    k0, v0, U = rand(n, Hkv, cap, dh), rand(n, Hkv, cap, dh), rand(n, P, Hq * dh)
+    sc = ph.make_layer_scratch(T, Hq, Hkv, dh, 128, "cuda", torch.bfloat16)
+    with Ctx(cfg, max_queries=T) as c:
+        k, v, ln, y = k0.clone(), v0.clone(), len0.clone(), torch.empty_like(U)
+        ph.photon_decoder_prefill(c.h, layer, sc, U, ph.make_kv(k, v, ln), ids, y, scale=scale)
+        assert c.status() == ph.PHOTON_DEV_CAPACITY
+        t = sc.tensors
+        q, kn, vn = torch.empty_like(t["q"]), torch.empty_like(t["k_new"]), torch.empty_like(t["v_new"])
+        ph.photon_rope_split(c.h, t["qkv"], torch.arange(P, dtype=torch.int32, device="cuda").repeat(n), q, kn, vn)
+        k1, v1, ln1, att = k0.clone(), v0.clone(), len0.clone(), torch.empty_like(t["att"])
+        kv1 = ph.make_kv(k1, v1, ln1)
+        ph.photon_kv_append(c.h, kv1, kn.view(n, P, Hkv, dh), vn.view(n, P, Hkv, dh), ids, n, P)
+        ph.photon_chunk_causal_attn(c.h, kv1, q.view(n, P, Hq, dh), ids, att.view(n, P, Hq, dh), n, 0, P, scale)
+        assert c.status() == ph.PHOTON_DEV_CAPACITY
+        for a, b in ((t["q"], q), (t["k_new"], kn), (t["v_new"], vn), (k, k1), (v, v1), (t["att"], att)):
+            assert np.array_equal(host_bits(a), host_bits(b))
+        assert torch.equal(ln, ln1)

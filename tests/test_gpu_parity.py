@@ -322,7 +322,7 @@ def test_converter_matches_oracle(oracle, idx, rows, layout):
 
 
 def test_converter_for_thousands_of_latents(oracle):
-    """A batch large enough for the persistent large-tile kernel (more than two tiles of
+    """A batch large enough for the persistent kernel of CTA pairs (more than two tiles of
     128 x 256 per SM), ragged last row tile, with bias; the oracle recomputes a sample of rows."""
     cfg = cfg_small(4, B=5000)                                  # D 1024, P 8: 40 x 32 tiles
     cv = wl.converter_inputs(cfg, with_bias=True)
