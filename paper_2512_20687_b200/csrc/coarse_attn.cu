@@ -54,7 +54,7 @@ constexpr int CTAS_PER_SM = 2;
 //    64 of 16 in four parts each 12.2 and 15.3;
 //  - with different lengths, 4 heads and 4 to 10 tiles per CTA (below, the length of the longest share is what counts), streams of at most 7 tiles more than the even share that are not close to
 //    it (a CTA gets two of those or none; 300 of 11 to 13 tiles, even share 12.5: 25.1 and 27.8 us); boundaries within 2 tiles of an end of
-//    another stream move there.  75 sequences of 0 to 1000 rows 20.6 -> 18.1 us, 32 of 0 to 1800 18.9 -> 16.9;
+//    another stream move there.  75 sequences of 0 to 1000 rows 22.1 -> 18.4 us, 32 of 0 to 1600 15.9 -> 13.9;
 //  - with different lengths and 8 heads or more, streams that are much longer or much shorter than the even share; ends likewise.
 template <int DH, int GP>
 struct Cuts {
