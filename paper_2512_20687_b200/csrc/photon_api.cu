@@ -36,17 +36,9 @@ bool kv_ok(const photon_ctx *ctx, const photon_kv *c, bool allow_shared) {
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 
-// k_new, v_new: the step's append folded into the attention over the units' own keys (see AttnParams), or NULL.
-photon_status attention_common(photon_ctx *ctx, const photon_kv *cache, const photon_bf16 *q,
-                               const int32_t *slot, int n_q, photon_bf16 *out, float *lse,
-                               float scale, bool chunk, cudaStream_t st, const photon_bf16 *k_new = nullptr,
-                               const photon_bf16 *v_new = nullptr, bool over_bus = false, bool dependent = false,
-                               bool replayed_first = false) {
-    if (!ctx) return PHOTON_ERR_INVALID_ARG;
-    if (!kv_ok(ctx, cache, !chunk) || (chunk && cache->page_table)) return PHOTON_ERR_INVALID_ARG;
-    if (n_q < 0 || (n_q > 0 && (!q || !out))) return PHOTON_ERR_INVALID_ARG;
-    if (!aligned16(q) || !aligned16(out)) return PHOTON_ERR_INVALID_ARG;
-    if (!(scale == scale)) return PHOTON_ERR_INVALID_ARG;
+// What an attention call asks of its cache and its workspace: calls of several kernels look before their first launch.
+photon_status attention_check(const photon_ctx *ctx, const photon_kv *cache, int n_q, float scale, bool chunk) {
+    if (!kv_ok(ctx, cache, !chunk) || (chunk && cache->page_table) || n_q < 0 || !(scale == scale)) return PHOTON_ERR_INVALID_ARG;
     if (n_q == 0) return PHOTON_OK;
     const photon_config &c = ctx->cfg;
     // TMA row coordinates are 32-bit
@@ -55,6 +47,21 @@ photon_status attention_common(photon_ctx *ctx, const photon_kv *cache, const ph
     if (pool_rows >= (1ull << 31)) return PHOTON_ERR_UNSUPPORTED;
     if (cache->k_shared && (uint64_t)cache->n_shared * c.Hkv * cache->cap_shared >= (1ull << 31))
         return PHOTON_ERR_UNSUPPORTED;
+    if (!chunk && (size_t)n_q * c.Hkv > ctx->n_tickets) return PHOTON_ERR_WORKSPACE;
+    if (!chunk && cache->k_shared && size_t(n_q) * c.Hq * (c.dh + 2) > ctx->partial_floats) return PHOTON_ERR_WORKSPACE;
+    return PHOTON_OK;
+}
+
+// k_new, v_new: the step's append folded into the attention over the units' own keys (see AttnParams), or NULL.
+photon_status attention_common(photon_ctx *ctx, const photon_kv *cache, const photon_bf16 *q,
+                               const int32_t *slot, int n_q, photon_bf16 *out, float *lse,
+                               float scale, bool chunk, cudaStream_t st, const photon_bf16 *k_new = nullptr,
+                               const photon_bf16 *v_new = nullptr, bool over_bus = false, bool dependent = false,
+                               bool replayed_first = false) {
+    if (!ctx || (n_q > 0 && (!q || !out)) || !aligned16(q) || !aligned16(out)) return PHOTON_ERR_INVALID_ARG;
+    if (const photon_status s = attention_check(ctx, cache, n_q, scale, chunk)) return s;
+    if (n_q == 0) return PHOTON_OK;
+    const photon_config &c = ctx->cfg;
     AttnParams p{};
     p.q = reinterpret_cast<const bf16 *>(q);
     p.out = reinterpret_cast<bf16 *>(out);
@@ -89,14 +96,12 @@ photon_status attention_common(photon_ctx *ctx, const photon_kv *cache, const ph
     p.max_len = cache->max_len ? cache->max_len : cache->cap;
     p.splits_sh = 0;
     if (!chunk) {
-        if ((size_t)n_q * c.Hkv > ctx->n_tickets) return PHOTON_ERR_WORKSPACE;
         if (cache->k_shared) {
             p.ks = reinterpret_cast<const bf16 *>(cache->k_shared);
             p.vs = reinterpret_cast<const bf16 *>(cache->v_shared);
             p.sh_len = cache->shared_len; p.sh_id = cache->shared_id;
             p.n_shared = cache->n_shared; p.cap_sh = cache->cap_shared;
             const int ms = cache->max_shared_len ? cache->max_shared_len : cache->cap_shared;
-            if (size_t(n_q) * c.Hq * (c.dh + 2) > ctx->partial_floats) return PHOTON_ERR_WORKSPACE;
             const int G = c.Hq / c.Hkv;
             const int groups = ceil_div(n_q, shared_prefix_units_per_cta(G));     // tiles of 128 query rows
             // key ranges per row tile = cluster size: a power of two up to 8, about one wave of CTAs in all
@@ -460,8 +465,8 @@ photon_status layer_step(photon_ctx *ctx, const photon_layer *L, const photon_la
     for (const void *q : ptrs)
         if (!q || !aligned16(q)) return PHOTON_ERR_INVALID_ARG;
     const int B = cache->n_units, D = c.D, QKV = (c.Hq + 2 * c.Hkv) * c.dh;
-    if (!local && (size_t)B * c.Hkv > ctx->n_tickets) return PHOTON_ERR_WORKSPACE;
-    if (local && (cache->cap > c.P + c.C || cache->page_table)) return PHOTON_ERR_INVALID_ARG;
+    if (local && cache->cap > c.P + c.C) return PHOTON_ERR_INVALID_ARG;
+    if (const photon_status bad = attention_check(ctx, cache, B, scale, local)) return bad;
     photon_status s = photon_rmsnorm(ctx, x, L->g1, L->eps, sc->n, B, D, stream);
     // Many chunks: the projection's epilogue rotates, splits and appends, and the projection itself (sc->qkv, 100 MB written and read
     // back with 16384 chunks of width 1024) is not written: projection and split 127 us, 75 so.  Few: a cut into whole heads costs
@@ -519,6 +524,7 @@ photon_status photon_decoder_prefill(photon_ctx *ctx, const photon_layer *L, con
     for (const void *q : ptrs)
         if (!q || !aligned16(q)) return PHOTON_ERR_INVALID_ARG;
     if (n == 0) return PHOTON_OK;
+    if (!(scale == scale)) return PHOTON_ERR_INVALID_ARG;
     const int P = c.P, T = n * P, D = c.D;                                       // T rows: the P prefix vectors of n chunks
     photon_status s = photon_rmsnorm(ctx, U, L->g1, L->eps, sc->n, T, D, stream);
     // one projection that rotates, splits and appends, instead of three kernels (a trip between kernels each; 64 chunks of 4 rows, 2048
@@ -615,7 +621,9 @@ photon_status step_impl(photon_ctx *ctx, const photon_step_args *a, photon_strea
             return PHOTON_ERR_INVALID_ARG;
         if (a->chunks->cap > c.P + c.C || (!a->slot && a->Nc > a->chunks->n_units))
             return PHOTON_ERR_INVALID_ARG;
+        if (const photon_status bad = attention_check(ctx, a->chunks, a->Nc, a->scale_chunk, true)) return bad;
     }
+    if (const photon_status bad = attention_check(ctx, a->coarse, a->coarse->n_units, a->scale_coarse, false)) return bad;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // The chunk attention shares no data with the other parts (the decoders' projections, which are not
     // built, sit between the converter's output and the chunk caches): it runs beside them on a

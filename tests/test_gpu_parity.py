@@ -887,3 +887,66 @@ def test_invalid_arguments_launch_nothing():
     with pytest.raises(ph.PhotonError) as e:
         ph.photon_create(4, 2, 96, 256, 4, 4, 16)
     assert e.value.code == ph.PHOTON_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("what", ["chunk scale", "coarse scale", "paged chunks", "workspace"])
+@pytest.mark.parametrize("captured", [False, True])
+def test_steps_that_are_refused_have_launched_nothing(what, captured):
+    """Whatever order a step's kernels are enqueued in (in line, beside, captured): a step that returns an error leaves the coarse cache,
+    the lengths and the outputs as they were."""
+    Hq, Hkv, dh, P, C, B, S, Nc = 4, 2, 64, 4, 60, 6, 64, 8
+    D = Hq * dh
+    cfg = wl.scaled(wl.CONFIGS[0], B=B, Hq=Hq, Hkv=Hkv, dh=dh, D=D, P=P, C=C)
+    new = lambda *s: torch.zeros(*s, dtype=torch.bfloat16, device="cuda")
+    k, v, ln = new(B, Hkv, S, dh), new(B, Hkv, S, dh), dev_i32(np.full(B, 20))
+    q, rows, out, U = new(B, Hq, dh) + 1, new(B, Hkv, dh) + 1, new(B, Hq, dh) + 7, new(B, P, D) + 7
+    qc, oc, w = new(Nc, Hq, dh) + 1, new(Nc, Hq, dh) + 7, new(D, P * D)
+    nan = float("nan")
+    if what == "paged chunks":
+        pool = new(Nc, Hkv, 64, dh)
+        ckv = ph.make_kv(pool, pool.clone(), dev_i32(np.full(Nc, P)), page_table=torch.arange(Nc, dtype=torch.int32, device="cuda").view(Nc, 1))
+    else:
+        ckv = ph.make_kv(new(Nc, Hkv, P + C, dh), new(Nc, Hkv, P + C, dh), dev_i32(np.full(Nc, P)))
+    with Ctx(cfg, max_queries=2 if what == "workspace" else Nc) as c:
+        args = ph.make_step_args(ph.make_kv(k, v, ln), rows, rows, q, out, nan if what == "coarse scale" else 1.0, w, ph.PHOTON_W_IN_MAJOR, U, B,
+                                 chunks=ckv, q_chunk=qc, out_chunk=oc, Nc=Nc, scale_chunk=nan if what == "chunk scale" else 1.0)
+        n0 = ph.photon_launch_count(c.h)
+        torch.cuda.synchronize()
+        if captured:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                with pytest.raises(ph.PhotonError):
+                    ph.photon_decode_step(c.h, args)
+                ln.add_(0)                                                # (a graph of something)
+            graph.replay()
+            del graph
+        else:
+            with pytest.raises(ph.PhotonError):
+                ph.photon_decode_step(c.h, args)
+        assert ph.photon_launch_count(c.h) == n0 and c.status() == 0
+        assert bool((ln == 20).all()) and not bool(k.any()) and not bool(v.any())
+        for t in (out, U, oc):
+            assert bool((t == 7).all())
+
+
+@pytest.mark.parametrize("call", ["encoder", "decoder", "prefill"])
+def test_layers_that_are_refused_have_launched_nothing(call):
+    Hq, Hkv, dh, P, C, n, F = 4, 2, 64, 4, 4, 6, 128
+    D = Hq * dh
+    cfg = wl.scaled(wl.CONFIGS[0], B=n, Hq=Hq, Hkv=Hkv, dh=dh, D=D, P=P, C=C)
+    new = lambda *s: torch.zeros(*s, dtype=torch.bfloat16, device="cuda")
+    layer = ph.make_layer(new(D), new(D, (Hq + 2 * Hkv) * dh), new(D, D), new(D), new(D, 2 * F), new(F, D), ph.PHOTON_W_IN_MAJOR, F)
+    sc = ph.make_layer_scratch(n * P, Hq, Hkv, dh, F, "cuda", torch.bfloat16)
+    k, v, ln = new(n, Hkv, P + C, dh) + 3, new(n, Hkv, P + C, dh) + 3, dev_i32(np.zeros(n))
+    kv, x, y = ph.make_kv(k, v, ln), new(n, P, D), new(n, P, D) + 7
+    with Ctx(cfg, max_queries=n) as c:
+        n0 = ph.photon_launch_count(c.h)
+        with pytest.raises(ph.PhotonError):
+            if call == "encoder":
+                ph.photon_encoder_step(c.h, layer, sc, x, kv, y, scale=float("nan"))
+            elif call == "decoder":
+                ph.photon_decoder_step(c.h, layer, sc, x, kv, y, scale=float("nan"))
+            else:
+                ph.photon_decoder_prefill(c.h, layer, sc, x, kv, None, y, n=n, scale=float("nan"))
+        assert ph.photon_launch_count(c.h) == n0 and c.status() == 0
+        assert bool((ln == 0).all()) and bool((k == 3).all()) and bool((v == 3).all()) and bool((y == 7).all())
